@@ -6,12 +6,13 @@
 //                h_{M/2} = 0), inverse FFT, crop to N samples.
 //   k_ss_bp      Eq. 2 as a Riemann sum: b[r][c] = sum_j w_j y_j(i_f) with
 //                i_f = (c - N/2) cos t_j + (r - N/2) sin t_j + N/2 and linear
-//                interpolation (zero outside [0, N-1]).  One 16 x 16 pixel tile
-//                and Q slices per block (the Q slices share the geometry, as the
-//                paper's blocks of Q sinograms do); batches of angles are staged
-//                in shared memory with zero fill, so the inner loop has no bounds
-//                tests.  The tile origin's detector coordinate is computed in
-//                double precision, the per-pixel offset (< 25 samples) in float.
+//                interpolation (zero outside [0, N-1]).  A tile of 32 columns
+//                and 4 or 16 rows and 4 or 8 slices per block (the slices share
+//                the geometry, as the paper's blocks of Q sinograms do); batches
+//                of angles are staged in shared memory with zero fill, so the
+//                inner loop has no bounds tests.  The tile centre's detector
+//                coordinate is computed in double precision, the per-pixel
+//                offset from it (< 18 samples) in float.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -94,74 +95,184 @@ __global__ void __launch_bounds__(TPL * LPC)
     fft_line<M, TPL, true>(t, sm, dst, sm, tw);
 }
 
-constexpr int SS_TILE = 16;
-constexpr int SS_AB = 16;   // angles per staged batch
-constexpr int SS_W = 28;    // staged samples per angle and slice (>= 15 (|cos| + |sin|) + 4)
+constexpr int SS_TX = 32;      // pixels of a tile along x (a warp's lanes)
+constexpr int SS_WARPS = 4;    // warps a block; warp w covers rows w R .. w R + R - 1 of the tile
+constexpr int SS_AB = 12;      // angles per staged batch
 
-template <int Q>
-__global__ void __launch_bounds__(256)
+// staged samples per angle and slice: 31 |cos| + (4 R - 1) sin + the window
+template <int R> __host__ __device__ constexpr int ss_w() { return R > 1 ? 40 : 36; }
+
+// acc += w * z for the 4 H slices, with packed FP32 multiply-adds (one issue
+// slot for two)
+template <int H>
+__device__ __forceinline__ void fma_slices(float2 (&acc)[H][2], float w, const float4 (&z)[H]) {
+    const float2 ww = make_float2(w, w);
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        acc[h][0] = __ffma2_rn(ww, make_float2(z[h].x, z[h].y), acc[h][0]);
+        acc[h][1] = __ffma2_rn(ww, make_float2(z[h].z, z[h].w), acc[h][1]);
+    }
+}
+
+// A thread holds R vertically adjacent pixels of 4 H slices.  Their detector
+// coordinates v_p = v_0 + p sin t (0 <= sin t <= 1) lie in
+// [floor(v_0), floor(v_0) + p + 1), so the samples floor(v_0) .. floor(v_0) + R
+// serve all R of them: sample k weighs max(0, 1 - |v_p - k|), which is linear
+// interpolation, and is zero for k > p + 1.  Each sample is read once per R
+// pixels, four slices to a 16-byte load (lanes along x read consecutive
+// 16-byte words: no bank conflicts): per pixel, angle and 8 slices 8.6
+// shared-memory wavefronts on average with R = 4 against 16 for two reads per
+// pixel and slice.  A batch of angles with a value that is not finite reads the
+// two samples of each pixel instead (a zero weight would not hide it).  What
+// bounds it: FP32 issue and the shared-memory wavefronts, about alike.  At
+// 512 x 512, 512 angles, 16 slices: 1033 us for the form with one pixel a
+// thread, two 4-byte loads a slice and 103 warp instructions per 32 pixels,
+// angle and 8 slices; 632 us with this one.
+template <int H, int R>
+__global__ void __launch_bounds__(32 * SS_WARPS, R > 1 ? 7 : 8)
     k_ss_bp(const float* __restrict__ y, int S, int V, int N, const double2* __restrict__ cs64,
             const float2* __restrict__ cs32, const float* __restrict__ wq, float* __restrict__ vol) {
-    __shared__ float seg[SS_AB][Q][SS_W];
-    __shared__ float bfrac[SS_AB];
-    __shared__ int blo[SS_AB];
-    __shared__ float2 bcs[SS_AB];
-    __shared__ float bw[SS_AB];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int c0 = blockIdx.x * SS_TILE, r0 = blockIdx.y * SS_TILE;
-    const int s0 = blockIdx.z * Q;
-    float acc[Q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) acc[q] = 0.f;
-    for (int jb = 0; jb < V; jb += SS_AB) {
-        __syncthreads();
-        if (threadIdx.x < SS_AB) {
-            const int j = jb + threadIdx.x;
-            if (j < V) {
-                const double2 cs = cs64[j];
-                const double fo = (double)(c0 - N / 2) * cs.x + (double)(r0 - N / 2) * cs.y + (double)(N / 2);
-                const double mn = fo + fmin(0.0, (SS_TILE - 1) * cs.x) + fmin(0.0, (SS_TILE - 1) * cs.y);
-                const int lo = (int)floor(mn) - 1;
-                blo[threadIdx.x] = lo;
-                bfrac[threadIdx.x] = (float)(fo - (double)lo);
-                bcs[threadIdx.x] = cs32[j];
-                bw[threadIdx.x] = wq[j];
-            }
+    constexpr int W = ss_w<R>();
+    constexpr int TY = SS_WARPS * R;
+    __shared__ float4 seg[SS_AB][H][W];
+    // per angle of the batch (double-buffered): cos, sin, fraction of the tile
+    // centre's coordinate, weight; staged index of its integer part (low half)
+    // and the last sample after floor(v_0) that a pixel can reach (high half),
+    // first staged sample
+    __shared__ float4 ang[2][SS_AB];
+    __shared__ int2 pos[2][SS_AB];
+    // the sums over the batches so far: a batch's sum starts at zero and is
+    // added once, so that rounding does not grow with the number of angles
+    __shared__ float4 total[R * H][32 * SS_WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c0 = blockIdx.x * SS_TX, r0 = blockIdx.y * TY;
+    const int s0 = blockIdx.z * (4 * H);
+    auto geometry = [&](int buf, int jb) {
+        const int j = jb + threadIdx.x;
+        if (threadIdx.x < SS_AB && j < V) {
+            const double2 cs = cs64[j];
+            const double fc = (double)(c0 + SS_TX / 2 - N / 2) * cs.x + (double)(r0 + TY / 2 - N / 2) * cs.y +
+                              (double)(N / 2);
+            const double mn = fc - (SS_TX / 2) * cs.x - (TY / 2) * cs.y + fmin(0.0, (SS_TX - 1) * cs.x);
+            const int lo = (int)floor(mn) - 1, ic = (int)floor(fc);
+            const float2 cf = cs32[j];
+            ang[buf][threadIdx.x] = make_float4(cf.x, cf.y, (float)(fc - (double)ic), wq[j]);
+            // pixel R - 1 lies below 1 + (R - 1) sin t; one more for its second sample
+            const int top = R == 1 ? 1 : 2 + (int)((float)(R - 1) * cf.y);
+            pos[buf][threadIdx.x] = make_int2((ic - lo) | (top << 16), lo);
         }
-        __syncthreads();
-        for (int e = threadIdx.x; e < SS_AB * Q * SS_W; e += 256) {
-            const int a = e / (Q * SS_W);
-            const int rem = e - a * (Q * SS_W);
-            const int qq = rem / SS_W, w = rem - qq * SS_W;
-            const int j = jb + a, s = s0 + qq;
-            float v = 0.f;
-            if (j < V && s < S) {
-                const int i = blo[a] + w;
-                if (i >= 0 && i < N) v = __ldg(y + ((size_t)s * V + j) * N + i) * bw[a];
-            }
-            seg[a][qq][w] = v;
-        }
-        __syncthreads();
+    };
+    const float fx = (float)(lane - SS_TX / 2), fy = (float)(warp * R - TY / 2);
+    geometry(0, 0);
+    for (int jb = 0, buf = 0; jb < V; jb += SS_AB, buf ^= 1) {
+        __syncthreads();   // this batch's geometry is there, the previous batch's samples are done with
         const int na = min(SS_AB, V - jb);
-        for (int a = 0; a < na; ++a) {
-            const float2 cs = bcs[a];
-            const float v = fmaf((float)tx, cs.x, fmaf((float)ty, cs.y, bfrac[a]));
-            const float fl = floorf(v);
-            const int i0 = (int)fl;
-            const float f = v - fl;
+        bool odd = false;   // a staged value is not finite
+        for (int a = warp; a < na; a += SS_WARPS) {
+            const int lo = pos[buf][a].y;
+            const float w = ang[buf][a].w;
+            const float* yj = y + (size_t)(jb + a) * N;
 #pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const float y0 = seg[a][q][i0], y1 = seg[a][q][i0 + 1];
-                acc[q] += fmaf(f, y1 - y0, y0);
+            for (int it = lane; it < H * W; it += 32) {
+                const int h = it >= W, i = it - h * W;
+                const int g = lo + i;
+                float v[4] = {0.f, 0.f, 0.f, 0.f};
+                if (g >= 0 && g < N) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int s = s0 + 4 * h + q;
+                        if (s < S) v[q] = __ldg(yj + (size_t)s * V * N + g) * w;
+                    }
+                }
+                seg[a][h][i] = make_float4(v[0], v[1], v[2], v[3]);
+                odd |= !(fabsf(v[0]) + fabsf(v[1]) + fabsf(v[2]) + fabsf(v[3]) < INFINITY);
+            }
+        }
+        geometry(buf ^ 1, jb + SS_AB);
+        odd = __syncthreads_or(odd);
+        float2 acc[R][H][2];
+#pragma unroll
+        for (int p = 0; p < R; ++p)
+#pragma unroll
+            for (int h = 0; h < H; ++h) acc[p][h][0] = acc[p][h][1] = make_float2(0.f, 0.f);
+        if (R > 1 && odd) {
+#pragma unroll 1
+            for (int a = 0; a < na; ++a) {
+                const float4 an = ang[buf][a];
+                const float vx = fmaf(fx, an.x, an.z);
+#pragma unroll
+                for (int p = 0; p < R; ++p) {
+                    const float v = fmaf(fy + (float)p, an.y, vx), fl = floorf(v);
+                    const float4* base = &seg[a][0][(int)fl + (pos[buf][a].x & 0xffff)];
+                    float4 z0[H], z1[H];
+#pragma unroll
+                    for (int h = 0; h < H; ++h) {
+                        z0[h] = base[h * W];
+                        z1[h] = base[h * W + 1];
+                    }
+                    fma_slices<H>(acc[p], 1.f - (v - fl), z0);
+                    fma_slices<H>(acc[p], v - fl, z1);
+                }
+            }
+        } else {
+            for (int a = 0; a < na; ++a) {
+                const float4 an = ang[buf][a];
+                const int ps = pos[buf][a].x;
+                const float vx = fmaf(fx, an.x, an.z);
+                const float v0 = fmaf(fy, an.y, vx);
+                const float fl = floorf(v0);
+                const float4* base = &seg[a][0][(int)fl + (ps & 0xffff)];
+                float d[R];   // coordinates from sample floor(v_0)
+                d[0] = v0 - fl;
+#pragma unroll
+                for (int p = 1; p < R; ++p) d[p] = fmaf(fy + (float)p, an.y, vx) - fl;
+#pragma unroll
+                for (int k = 0; k <= R; ++k) {
+                    if (k > 2 && k > ps >> 16) break;   // the same for the whole block
+                    float4 z[H];
+#pragma unroll
+                    for (int h = 0; h < H; ++h) z[h] = base[h * W + k];
+#pragma unroll
+                    for (int p = k > 1 ? k - 1 : 0; p < R; ++p)
+                        fma_slices<H>(acc[p],
+                                      k == 0 ? __saturatef(1.f - d[p]) : __saturatef(1.f - fabsf(d[p] - (float)k)), z);
+                }
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < R; ++p)
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                float4& t = total[p * H + h][threadIdx.x];   // this thread's own
+                const float2 lo = acc[p][h][0], hi = acc[p][h][1];
+                const float4 o = jb ? t : make_float4(0.f, 0.f, 0.f, 0.f);
+                t = make_float4(o.x + lo.x, o.y + lo.y, o.z + hi.x, o.w + hi.y);
+            }
+    }
+    const int c = c0 + lane;
+#pragma unroll
+    for (int p = 0; p < R; ++p) {
+        const int r = r0 + warp * R + p;
+        if (r < N && c < N) {
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                const float4 t = total[p * H + h][threadIdx.x];
+                const float v[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int s = s0 + 4 * h + q;
+                    if (s < S) vol[((size_t)s * N + r) * N + c] = v[q];
+                }
             }
         }
     }
-    const int r = r0 + ty, c = c0 + tx;
-    if (r < N && c < N) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q)
-            if (s0 + q < S) vol[((size_t)(s0 + q) * N + r) * N + c] = acc[q];
-    }
+}
+
+template <int H, int R>
+static void launch_ss_bp(const bst_plan_s* p, const float* y, int slices, float* vol, cudaStream_t st) {
+    const int N = p->N;
+    const dim3 grid((N + SS_TX - 1) / SS_TX, (N + SS_WARPS * R - 1) / (SS_WARPS * R), (slices + 4 * H - 1) / (4 * H));
+    k_ss_bp<H, R><<<grid, 32 * SS_WARPS, 0, st>>>(y, slices, p->V, N, p->cs64, p->cs32, p->wq, vol);
 }
 
 template <int M>
@@ -211,11 +322,18 @@ bst_status_t bst_launch_brute(bst_plan_s* p, const float* sino, int slices, cons
         if (s != BST_OK) return s;
         y = q;
     }
-    constexpr int Q = 8;
-    const int N = p->N;
-    dim3 grid((N + bst::SS_TILE - 1) / bst::SS_TILE, (N + bst::SS_TILE - 1) / bst::SS_TILE, (slices + Q - 1) / Q);
+    // Four pixels a thread where that still gives every SM a few blocks; one
+    // pixel a thread (four times the blocks) where it does not, and four slices
+    // a thread where there are no more.
+    const long long blocks4 = (long long)((p->N + 31) / 32) * ((p->N + 15) / 16) * ((slices + 7) / 8);
     bst_timing_mark(p, st, -1);
-    bst::k_ss_bp<Q><<<grid, 256, 0, st>>>(y, slices, p->V, N, p->cs64, p->cs32, p->wq, vol);
+    if (slices > 4) {
+        if (blocks4 >= 304) bst::launch_ss_bp<2, 4>(p, y, slices, vol, st);
+        else bst::launch_ss_bp<2, 1>(p, y, slices, vol, st);
+    } else {
+        if (blocks4 >= 304) bst::launch_ss_bp<1, 4>(p, y, slices, vol, st);
+        else bst::launch_ss_bp<1, 1>(p, y, slices, vol, st);
+    }
     bst_timing_mark(p, st, 4);
     return cudaGetLastError() == cudaSuccess ? BST_OK : BST_ERR_CUDA;
 }
