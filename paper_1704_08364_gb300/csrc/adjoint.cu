@@ -8,7 +8,8 @@
 //   k_adj_row_fft   transpose of the crop and the row inverse FFT: zero-extend
 //                   each image row to M and FFT it (opposite exponent).
 //   k_adj_col_fft   transpose of the column inverse FFT: zero-extend each
-//                   column to M and FFT it, giving the full Cartesian spectrum.
+//                   column to M and FFT it, giving the full Cartesian spectrum,
+//                   up to four slice pairs interleaved point by point.
 //   k_adj_polar     transpose of the bilinear gridding in gather form: every
 //                   polar sample (j, k) sums the weighted Cartesian values of
 //                   the gridding cells that tap it (cell lists built once per
@@ -18,22 +19,41 @@
 //                   the inverse FFT along t, cropped to the N detector samples,
 //                   scaled by dt dw^2, Re -> slice a, Im -> slice b.
 //
-// The filter gradient recomputes the ray spectrum Y (no weight) and the
-// polar pull-back lambda of the image gradient, and reduces
-// Re(conj(lambda) Y) over angles, slices and +-k in a fixed order.
+// The filter gradient multiplies the rays' spectrum Y (no weight), recomputed
+// block by block (k_fg_ray), by the polar pull-back lambda of the image
+// gradient, and reduces Re(conj(lambda) Y) over angles, slices and +-k in a
+// fixed order.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
+#include <cstdint>
 #include <vector>
 
-#include "bst_fft.cuh"
-#include "bst_geo.cuh"
-#include "bst_internal.h"
+#include "bst_stages.cuh"
 
 namespace bst {
 
 template <int M> __host__ __device__ constexpr int adj_tpl() { return (M % 3 == 0) ? M / 12 : M / 16; }
 template <int M> __host__ __device__ constexpr int adj_row_stride() { return smem_line_len(M) + 4; }
+// most slice pairs whose spectra are interleaved: four lines of 256 threads at
+// M = 4096 would leave one block an SM
+template <int M> __host__ __device__ constexpr int adj_pairs() { return M >= 3072 ? 2 : 4; }
+// lines (columns times P pairs) of a block of the column kernel: 256 threads or
+// more
+template <int M, int P> __host__ __device__ constexpr int adj_col_lines() {
+    const int n = 256 / (adj_tpl<M>() * P);
+    return n > 1 ? n * P : P;
+}
+// lines (angle rows times P pairs) of a block of the polar kernel: its threads
+// walk the rows one after the other, so four rows at most (more only to fill a
+// warp)
+template <int M, int P> __host__ __device__ constexpr int adj_polar_lines() {
+    const int warp = 32 / (adj_tpl<M>() * P), n = 256 / (adj_tpl<M>() * P);
+    const int rows = n > 4 ? 4 : n;
+    const int l = warp > rows ? warp : rows;
+    return l > 1 ? l * P : P;
+}
 
 // ---------------------------------------------------------------------------
 // k_adj_row_fft
@@ -88,35 +108,43 @@ __global__ void __launch_bounds__(4 * TPL * TPC)
 struct TileColSrc {
     const float2* T;
     int N, M, cidx;
+    bool live;
     static constexpr bool kSmem = false;
     __device__ __forceinline__ float2 load(int p) const {
         const int r = signed_freq(p, M) + (N >> 1);
-        if (r < 0 || r >= N) return make_float2(0.f, 0.f);
+        if (!live || r < 0 || r >= N) return make_float2(0.f, 0.f);
         return __ldg(T + ((size_t)(r >> 2) * M + cidx) * 4 + (r & 3));
     }
 };
 
 struct ColOut {
-    float2* X;
+    float2* X;     // the column, of this pair among P
+    int P;
     bool live;
     static constexpr bool kSmem = false;
     __device__ __forceinline__ void store(int k, float2 v) const {
-        if (live) X[k] = v;
+        if (live) X[(size_t)k * P] = v;
     }
 };
 
-template <int M, int TPL, int LPC>
-__global__ void __launch_bounds__(TPL * LPC)
-    k_adj_col_fft(const float2* __restrict__ T, int N, float2* __restrict__ X, const float2* __restrict__ tw) {
+// The spectra of P slice pairs interleaved, X[group][c][r][P], so that the
+// polar kernel reads a Cartesian point of all P pairs as one 8 P byte piece.
+// Lane order: pair, then position, so that the stores of a warp are contiguous;
+// the pairs' lines are skewed by 32 / P banks.  Pairs beyond npairs are zero.
+template <int M, int P> __host__ __device__ constexpr int adj_col_stride() {
+    return smem_line_len(M) + (P > 1 ? 16 / P : 0);
+}
+template <int M, int TPL, int LINES, int P>
+__global__ void __launch_bounds__(TPL * LINES)
+    k_adj_col_fft(const float2* __restrict__ T, int N, int npairs, float2* __restrict__ X,
+                  const float2* __restrict__ tw) {
     extern __shared__ float2 smem[];
-    const int pl = blockIdx.y;
-    const int line = threadIdx.x / TPL, t = threadIdx.x % TPL;
-    const int c = blockIdx.x * LPC + line;
-    const bool live = c < M;
-    const int cc = live ? c : 0;
-    TileColSrc src{T + (size_t)pl * ((N + 3) / 4) * 4 * M, N, M, cc};
-    ColOut dst{X + ((size_t)pl * M + cc) * M, live};
-    SmemLine sm{smem + line * smem_line_len(M)};
+    const int p = threadIdx.x % P, t = (threadIdx.x / P) % TPL, cl = threadIdx.x / (P * TPL);
+    const int pl = blockIdx.y * P + p;
+    const int c = blockIdx.x * (LINES / P) + cl;
+    TileColSrc src{T + (size_t)pl * ((N + 3) / 4) * 4 * M, N, M, c, pl < npairs && c < M};
+    ColOut dst{X + ((size_t)blockIdx.y * M + c) * M * P + p, P, c < M};
+    SmemLine sm{smem + (cl * P + p) * adj_col_stride<M, P>()};
     fft_line<M, TPL, false>(t, src, dst, sm, tw);
 }
 
@@ -129,68 +157,71 @@ struct Cells {
     const float2* __restrict__ w;    // (fth, fk) of each point
 };
 
-// Weighted sum of the Cartesian values of the cell (J, K0) for its tap `tap`
+// the values of P pairs at one Cartesian point
+template <int P>
+__device__ __forceinline__ void load_point(const float2* __restrict__ X, int pt, float2 (&x)[P]) {
+    if constexpr (P == 1) {
+        x[0] = __ldg(X + pt);
+    } else {
+        // (one 32-byte load for P = 4 measured slower: 358 against 280 us)
+        const float4* q = reinterpret_cast<const float4*>(X + (size_t)pt * P);
+#pragma unroll
+        for (int i = 0; i < P / 2; ++i) {
+            const float4 v = __ldg(q + i);
+            x[2 * i] = make_float2(v.x, v.y);
+            x[2 * i + 1] = make_float2(v.z, v.w);
+        }
+    }
+}
+
+template <int P>
+__device__ __forceinline__ void axpy(float2 (&acc)[P], float w, const float2 (&x)[P]) {
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        acc[p].x = fmaf(w, x[p].x, acc[p].x);
+        acc[p].y = fmaf(w, x[p].y, acc[p].y);
+    }
+}
+
+// acc += the weighted Cartesian values of the cell (J, K0) for its tap `tap`
 // (0: (J, K0), 1: (J, K0+1), 2: (J+1, K0), 3: (J+1, K0+1)).
-__device__ __forceinline__ float2 cell_sum(const Cells& cl, const float2* __restrict__ X, int M, int J, int K0,
-                                           int tap) {
-    float2 acc = make_float2(0.f, 0.f);
-    if (K0 < -(M >> 1) || K0 > (M >> 1) - 1) return acc;
+template <int P>
+__device__ __forceinline__ void add_cell(const Cells& cl, const float2* __restrict__ X, int M, int J, int K0, int tap,
+                                         float2 (&acc)[P]) {
+    if (K0 < -(M >> 1) || K0 > (M >> 1) - 1) return;
     const int cell = (J + 1) * M + (K0 + (M >> 1));
     const int b = __ldg(cl.start + cell), e = __ldg(cl.start + cell + 1);
     for (int i = b; i < e; ++i) {
         const float2 fw = __ldg(cl.w + i);
-        const float wt = (tap & 2 ? fw.x : 1.f - fw.x) * (tap & 1 ? fw.y : 1.f - fw.y);
-        const float2 x = __ldg(X + __ldg(cl.pts + i));
-        acc.x = fmaf(wt, x.x, acc.x);
-        acc.y = fmaf(wt, x.y, acc.y);
+        float2 x[P];
+        load_point<P>(X, __ldg(cl.pts + i), x);
+        axpy<P>(acc, (tap & 2 ? fw.x : 1.f - fw.x) * (tap & 1 ? fw.y : 1.f - fw.y), x);
     }
-    return acc;
 }
 
-// Weighted sum over the cells (J, K0 - 1) (tap `hi`: its radial weight is fk)
-// and (J, K0) (tap `lo`: 1 - fk), which are adjacent in the cell lists, with
-// angular weight fth (rows J + 1 of the bracket) or 1 - fth (row J).
-__device__ __forceinline__ float2 cell_pair_sum(const Cells& cl, const float2* __restrict__ X, int M, int J, int K0,
-                                                bool upper) {
-    float2 acc = make_float2(0.f, 0.f);
-    const int cell = (J + 1) * M + (K0 + (M >> 1));
-    const int b = __ldg(cl.start + cell - 1), mid = __ldg(cl.start + cell), e = __ldg(cl.start + cell + 1);
-    for (int i = b; i < e; ++i) {
-        const float2 fw = __ldg(cl.w + i);
-        const float wt = (upper ? fw.x : 1.f - fw.x) * (i < mid ? fw.y : 1.f - fw.y);
-        const float2 x = __ldg(X + __ldg(cl.pts + i));
-        acc.x = fmaf(wt, x.x, acc.x);
-        acc.y = fmaf(wt, x.y, acc.y);
+// First-pass source of the inverse FFT along t: lambda from the shared line
+// (plus the transpose of the mean at k = 0), kept in lam if asked for, times the
+// weight W of `mode`.
+struct PolarSrc {
+    const float2* p;
+    float2* lam;        // this pair's and angle's row, or null
+    const float* g;
+    float2 dc;          // spectrum value at (0, 0) / V
+    int M, mode;
+    float two_alpha;
+    static constexpr bool kSmem = true;
+    __device__ __forceinline__ float2 load(int k) const {
+        float2 v = p[k + (k >> 4)];
+        if (k == 0) v = cadd(v, dc);
+        if (lam) lam[k] = v;
+        const int ak = k <= (M >> 1) ? k : M - k;
+        float w;
+        if (ak == (M >> 1)) w = 0.f;
+        else if (mode == BSTK_FILTER) w = g ? __ldg(g + ak) : 1.f;
+        else w = ak == 0 ? 0.f : __fdiv_rn(two_alpha, (float)ak);
+        return cscale(v, w);
     }
-    return acc;
-}
-
-// lambda_j[K]: transpose of the gridding (every cell tap that lands on (j, K))
-__device__ __forceinline__ float2 polar_pullback(const Cells& cl, const float2* __restrict__ X, int V, int M, int j,
-                                                 int K) {
-    float2 s = make_float2(0.f, 0.f);
-    if (K <= -(M >> 1)) return s;
-    float2 v;
-    // taps (j, K) of the cells (j, K) [weight 1 - fk] and (j, K - 1) [weight fk], bracket row J = j
-    v = cell_pair_sum(cl, X, M, j, K, false);
-    s.x += v.x; s.y += v.y;
-    // the same from bracket J = j - 1, whose upper row J + 1 is j
-    v = cell_pair_sum(cl, X, M, j - 1, K, true);
-    s.x += v.x; s.y += v.y;
-    if (j == 0) {  // seam: the J+1 = V taps of bracket V-1 read row 0 at -k
-        v = cell_sum(cl, X, M, V - 1, -K, 2);
-        s.x += v.x; s.y += v.y;
-        v = cell_sum(cl, X, M, V - 1, -K - 1, 3);
-        s.x += v.x; s.y += v.y;
-    }
-    if (j == V - 1) {  // the J = -1 taps of bracket -1 read row V-1 at -k
-        v = cell_sum(cl, X, M, -1, -K, 0);
-        s.x += v.x; s.y += v.y;
-        v = cell_sum(cl, X, M, -1, -K - 1, 1);
-        s.x += v.x; s.y += v.y;
-    }
-    return s;
-}
+};
 
 struct SinoCrop {
     float* ya;
@@ -211,45 +242,118 @@ struct SinoCrop {
 // mode: BSTK_FILTER / BSTK_BACKPROJECT: weight, inverse FFT, crop -> sino;
 //       BSTK_RAW: no sinogram.
 // lam (may be null in the first two modes): lambda (no weight) to lam[pair][V][M]
-template <int M, int TPL, int LPC>
-__global__ void __launch_bounds__(TPL * LPC)
-    k_adj_polar(const float2* __restrict__ X, Cells cl, int V, int N, int slices, int pair0, int mode,
+//
+// A block takes L = LINES / P angle rows j0 .. of P slice pairs.  Thread kappa
+// walks the cells (J, K0 = kappa - M/2) of the brackets J = j0 - 1 .. j0 + L - 1
+// and reads each list entry and its P-pair point once for the four polar
+// samples it feeds: rows J and J + 1, bins K0 (its own) and K0 + 1 (handed to
+// the next lane by a shuffle, across warps through `edge`).  Reading every cell
+// once per sample and pair instead (four times, 8 bytes of each 32-byte sector)
+// waited on the list-to-point chains (16 stall cycles per issue): 486 us for
+// the 8 pairs of 16 x 1024 x 1024, 280 us with this form.  What bounds it
+// now is the latency and sector traffic of the point reads from L2.
+template <int M, int TPL, int LINES, int P>
+__global__ void __launch_bounds__(TPL * LINES, 1024 / (TPL * LINES))
+    k_adj_polar(const float2* __restrict__ X, Cells cl, int V, int N, int slices, int pair0, int npairs, int mode,
                 const float* __restrict__ g, float two_alpha, float scale, float* __restrict__ sino,
                 float2* __restrict__ lam, const float2* __restrict__ tw) {
+    constexpr int NT = TPL * LINES, L = LINES / P, H = M / 2;
+    constexpr int EDGES = (M - 1) / 32;   // warp boundaries within a row
+    static_assert(NT % 32 == 0 && LINES % P == 0, "whole warps, whole groups of pairs");
     extern __shared__ float2 smem[];
-    const int pl = blockIdx.y;
-    const int line = threadIdx.x / TPL, t = threadIdx.x % TPL;
-    const int j = blockIdx.x * LPC + line;
-    const bool live = j < V;
-    const int jj = live ? j : 0;
-    const float2* Xp = X + (size_t)pl * M * M;
-    const SmemLine sm{smem + line * smem_line_len(M)};
-    const float2 origin = __ldg(Xp);   // spectrum value at (0, 0)
-    for (int k = t; k < M; k += TPL) {
-        float2 v = make_float2(0.f, 0.f);
-        if (live) {
-            v = polar_pullback(cl, Xp, V, M, jj, signed_freq(k, M));
-            if (k == 0) {
-                v.x += origin.x / (float)V;
-                v.y += origin.y / (float)V;
+    __shared__ float2 edge[EDGES > 0 ? EDGES : 1][LINES];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int j0 = blockIdx.x * L;
+    const float2* Xp = X + (size_t)blockIdx.y * P * M * M;
+    const float2 zero = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int k0 = 0; k0 < M; k0 += NT) {
+        const int kappa = k0 + tid;
+        const bool act = kappa < M;
+        const int K = kappa - H;
+        float2 own[P], hi[P];   // of the row being completed, rows J + 1 of the brackets so far
+#pragma unroll
+        for (int p = 0; p < P; ++p) own[p] = hi[p] = zero;
+#pragma unroll 1
+        for (int b = 0; b <= L; ++b) {
+            const int J = j0 - 1 + b;
+            float2 own1[P], hi1[P];
+#pragma unroll
+            for (int p = 0; p < P; ++p) own1[p] = hi1[p] = zero;
+            if (act && J < V) {
+                const int cell = (J + 1) * M + kappa;
+                const int e = __ldg(cl.start + cell + 1);
+                for (int i = __ldg(cl.start + cell); i < e; ++i) {
+                    const float2 fw = __ldg(cl.w + i);
+                    float2 x[P];
+                    load_point<P>(Xp, __ldg(cl.pts + i), x);
+                    const float lo = 1.f - fw.x, l0 = 1.f - fw.y;
+                    axpy<P>(own, lo * l0, x);
+                    axpy<P>(hi, lo * fw.y, x);
+                    axpy<P>(own1, fw.x * l0, x);
+                    axpy<P>(hi1, fw.x * fw.y, x);
+                }
+            }
+            if (b > 0) {
+                const int j = J, l = b - 1;
+                if (act && j == 0) {  // seam: the J + 1 = V taps of bracket V - 1 read row 0 at -k
+                    add_cell<P>(cl, Xp, M, V - 1, -K, 2, own);
+                    add_cell<P>(cl, Xp, M, V - 1, -K - 1, 3, own);
+                }
+                if (act && j == V - 1) {  // the J = -1 taps of bracket -1 read row V - 1 at -k
+                    add_cell<P>(cl, Xp, M, -1, -K, 0, own);
+                    add_cell<P>(cl, Xp, M, -1, -K - 1, 1, own);
+                }
+                const int k = K < 0 ? K + M : K;
+#pragma unroll
+                for (int p = 0; p < P; ++p) {
+                    const int line = l * P + p;
+                    float2 up = make_float2(__shfl_up_sync(0xffffffffu, hi[p].x, 1),
+                                            __shfl_up_sync(0xffffffffu, hi[p].y, 1));
+                    if (lane == 0) up = zero;
+                    if (act) {
+                        // bin -M/2 is zero
+                        SmemLine{smem + line * smem_line_len(M)}.store(k, K == -H ? zero : cadd(own[p], up));
+                        if (lane == 31 && kappa + 1 < M) edge[kappa / 32][line] = hi[p];
+                    }
+                }
+            }
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                own[p] = own1[p];
+                hi[p] = hi1[p];
             }
         }
-        if (lam && live) lam[((size_t)pl * V + jj) * M + k] = v;
-        if (mode != BSTK_RAW) {
-            const int ak = k <= (M >> 1) ? k : M - k;
-            float w;
-            if (ak == (M >> 1)) w = 0.f;
-            else if (mode == BSTK_FILTER) w = g ? __ldg(g + ak) : 1.f;
-            else w = ak == 0 ? 0.f : __fdiv_rn(two_alpha, (float)ak);
-            sm.store(k, make_float2(v.x * w, v.y * w));
-        }
     }
-    if (mode == BSTK_RAW) return;   // uniform across the block
     __syncthreads();
+    for (int i = tid; i < EDGES * LINES; i += NT) {
+        const int line = i % LINES, w = i / LINES;
+        const int K = 32 * (w + 1) - H;
+        const int k = K < 0 ? K + M : K;
+        float2* q = smem + line * smem_line_len(M) + k + (k >> 4);
+        *q = cadd(*q, edge[w][line]);
+    }
+    __syncthreads();
+    const int line = tid / TPL, t = tid % TPL, p = line % P;
+    const int pl = blockIdx.y * P + p, j = j0 + line / P;
+    const bool live = j < V && pl < npairs;
+    const SmemLine sm{smem + line * smem_line_len(M)};
+    const float2 origin = __ldg(Xp + p);   // spectrum value at (0, 0)
+    const PolarSrc src{sm.p,
+                       lam && live ? lam + ((size_t)pl * V + j) * M : nullptr,
+                       g,
+                       make_float2(origin.x / (float)V, origin.y / (float)V),
+                       M,
+                       mode,
+                       two_alpha};
+    if (mode == BSTK_RAW) {   // uniform across the block
+        for (int k = t; k < M; k += TPL) src.load(k);
+        return;
+    }
     const int sa = 2 * (pair0 + pl), sb = sa + 1;
-    SinoCrop dst{sino + ((size_t)sa * V + jj) * N, sb < slices ? sino + ((size_t)sb * V + jj) * N : nullptr, N, M,
+    SinoCrop dst{sino + ((size_t)sa * V + j) * N, sb < slices ? sino + ((size_t)sb * V + j) * N : nullptr, N, M,
                  scale, live};
-    fft_line<M, TPL, true>(t, sm, dst, sm, tw);
+    fft_line<M, TPL, true>(t, src, dst, sm, tw);
 }
 
 // ---------------------------------------------------------------------------
@@ -277,49 +381,77 @@ __global__ void k_cell_keys(Geo geo, int M, int* __restrict__ key, float2* __res
 // ---------------------------------------------------------------------------
 // filter gradient reductions
 
-// part[pair][k] = sum_j Re(conj(lam_j[k]) Y_j[k])
-// part[pair][k] = sum_j Re(conj(lam_j[k]) Y_j[k]): a block takes 32 bins k and
-// splits the angles over 8 groups of its threads (j = g, g + 8, ...), whose
-// sums are then added in a fixed order (deterministic)
-constexpr int FG_K = 32, FG_G = 8;
-__global__ void __launch_bounds__(FG_K * FG_G)
-    k_fg_partial(const float2* __restrict__ lam, const float2* __restrict__ Y, int V, int M, int pair0,
-                 float* __restrict__ part) {
-    __shared__ float red[FG_G][FG_K];
-    const int kl = threadIdx.x % FG_K, grp = threadIdx.x / FG_K;
-    const int k = blockIdx.x * FG_K + kl;
+// part[pair JB + block][k] (+)= sum over the block's angles of Re(conj(lam_j[k]) Y_j[k]):
+// block x takes the groups of LPC angles x, x + JB, ..., transforms their padded
+// rays and multiplies by lambda while the spectrum is in shared memory, so Y
+// never goes to HBM.  Writing Y and reducing it in a second kernel took 54 +
+// 118 us for 16 x 1024 x 1024 (64 blocks a pair walking the angles: 12 %
+// occupancy), 65 us in this form.  Fixed order: deterministic.
+template <int M, int TPL, int LPC>
+__global__ void __launch_bounds__(TPL * LPC, (TPL * LPC <= 1024) ? 1024 / (TPL * LPC) : 1)
+    k_fg_ray(const float* __restrict__ sino, int slices, int pair0, int N, int V, const float2* __restrict__ lam,
+             int add, float* __restrict__ part, const float2* __restrict__ tw) {
+    extern __shared__ float2 smem[];
+    constexpr int PPT = M / TPL;
+    const int line = threadIdx.x / TPL, t = threadIdx.x % TPL;
     const int pl = blockIdx.y;
-    float s = 0.f;
-    if (k < M) {
-        const float2* l = lam + (size_t)pl * V * M + k;
-        const float2* y = Y + (size_t)pl * V * M + k;
-        for (int j = grp; j < V; j += FG_G) {
-            const float2 a = __ldg(l + (size_t)j * M), b = __ldg(y + (size_t)j * M);
-            s = fmaf(a.x, b.x, fmaf(a.y, b.y, s));
-        }
-    }
-    red[grp][kl] = s;
-    __syncthreads();
-    if (grp == 0 && k < M) {
-        float t = 0.f;
+    const int sa = 2 * (pair0 + pl), sb = sa + 1;
+    const SmemLine sm{smem + line * smem_line_len(M)};
+    float acc[PPT];
 #pragma unroll
-        for (int g = 0; g < FG_G; ++g) t += red[g][kl];
-        part[(size_t)(pair0 + pl) * M + k] = t;
+    for (int i = 0; i < PPT; ++i) acc[i] = 0.f;
+    for (int jb = blockIdx.x * LPC; jb < V; jb += gridDim.x * LPC) {
+        const int j = jb + line;
+        const bool live = j < V;
+        const int jj = live ? j : 0;
+        const RaySrc<0> src{sino + ((size_t)sa * V + jj) * N,
+                            sb < slices ? sino + ((size_t)sb * V + jj) * N : nullptr, N, M, live};
+        fft_line<M, TPL, false, 16, true>(t, src, sm, sm, tw);
+        __syncthreads();
+        const float2* l = lam + ((size_t)pl * V + jj) * M + t;
+#pragma unroll
+        for (int i = 0; i < PPT; ++i) {
+            const float2 a = __ldg(l + i * TPL), b = sm.load(t + i * TPL);   // b = 0 in a dead line
+            if (live) acc[i] = fmaf(a.x, b.x, fmaf(a.y, b.y, acc[i]));
+        }
+        __syncthreads();
+    }
+    float* red = reinterpret_cast<float*>(smem);
+#pragma unroll
+    for (int i = 0; i < PPT; ++i) red[line * M + t + i * TPL] = acc[i];
+    __syncthreads();
+    float* out = part + ((size_t)pl * gridDim.x + blockIdx.x) * M;
+    for (int k = threadIdx.x; k < M; k += TPL * LPC) {
+        float s = 0.f;
+#pragma unroll
+        for (int q = 0; q < LPC; ++q) s += red[q * M + k];
+        out[k] = add ? out[k] + s : s;
     }
 }
 
-// grad[m] = scale * sum over pairs of part[k = m] + part[k = M - m] (m = 1..M/2-1), fixed order;
-// scale = dt dw^2 restores the constants the unscaled transforms leave out
-__global__ void k_fg_final(const float* __restrict__ part, int pairs, int M, float scale, float* __restrict__ grad) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M / 2) return;
+// grad[m] = scale * sum over the rows of part of part[m] + part[M - m] (m = 1..M/2-1), fixed order;
+// scale = dt dw^2 restores the constants the unscaled transforms leave out.  A
+// block takes 32 bins and splits the rows over 32 groups of its threads.
+constexpr int FG_K = 32, FG_G = 32;
+__global__ void __launch_bounds__(FG_K * FG_G)
+    k_fg_final(const float* __restrict__ part, int rows, int M, float scale, float* __restrict__ grad) {
+    __shared__ float red[FG_G][FG_K];
+    const int kl = threadIdx.x % FG_K, grp = threadIdx.x / FG_K;
+    const int m = blockIdx.x * FG_K + kl;
     float s = 0.f;
-    for (int p = 0; p < pairs; ++p) {
-        const float* q = part + (size_t)p * M;
-        s += q[m];
-        if (m != 0) s += q[M - m];
+    if (m < M / 2)
+        for (int r = grp; r < rows; r += FG_G) {
+            const float* q = part + (size_t)r * M;
+            s += q[m] + (m != 0 ? q[M - m] : 0.f);
+        }
+    red[grp][kl] = s;
+    __syncthreads();
+    if (grp == 0 && m < M / 2) {
+        float t = 0.f;
+#pragma unroll
+        for (int q = 0; q < FG_G; ++q) t += red[q][kl];
+        grad[m] = t * scale;
     }
-    grad[m] = s * scale;
 }
 
 // ---------------------------------------------------------------------------
@@ -336,67 +468,117 @@ template <int M> struct AdjCfg {
     static constexpr int TPC = (128 / (4 * TPL)) > 1 ? 128 / (4 * TPL) : 1;
     static constexpr int LPC = (256 / TPL) > 1 ? 256 / TPL : 1;
     static constexpr size_t S1 = (size_t)4 * TPC * adj_row_stride<M>() * sizeof(float2);
-    static constexpr size_t S2 = (size_t)LPC * smem_line_len(M) * sizeof(float2);
+    static constexpr size_t SF = (size_t)LPC * smem_line_len(M) * sizeof(float2);
+    template <int P> static constexpr int LC = adj_col_lines<M, P>();
+    template <int P> static constexpr int LP = adj_polar_lines<M, P>();
+    template <int P> static constexpr size_t SC = (size_t)LC<P> * adj_col_stride<M, P>() * sizeof(float2);
+    template <int P> static constexpr size_t SP = (size_t)LP<P> * smem_line_len(M) * sizeof(float2);
 };
 
 struct AdjLayout {
-    int chunk;
-    float2 *T, *X, *lam, *Y;
+    int chunk;            // slice pairs in flight
+    int fg_blocks;        // angle blocks per pair of the filter gradient
+    float2 *T, *X, *lam;  // T and lam share their space: T is read before lam is written
     float* part;
 };
 
+static size_t adj_rows_t(const bst_plan_s* p) { return (size_t)((p->N + 3) / 4) * 4; }
+
 static size_t adj_bytes_per_pair(const bst_plan_s* p) {
-    const size_t rows_t = (size_t)((p->N + 3) / 4) * 4;
-    return (rows_t * p->M + (size_t)p->M * p->M + 2 * (size_t)p->V * p->M) * sizeof(float2);
+    return (std::max(adj_rows_t(p), (size_t)p->V) * p->M + (size_t)p->M * p->M) * sizeof(float2);
 }
 
+// Pairs in flight: as many as fit in 512 MiB, whole groups of four where there
+// are more, and at least the pairs that the polar kernel takes together.
 static int adj_chunk(const bst_plan_s* p, int pairs) {
-    const size_t budget = (size_t)256 << 20;
-    return (int)std::max<size_t>(1, std::min<size_t>((size_t)pairs, budget / adj_bytes_per_pair(p)));
+    const size_t budget = (size_t)512 << 20;
+    size_t c = std::max<size_t>(p->M >= 3072 ? 2 : 4, budget / adj_bytes_per_pair(p));
+    if (c > 4) c &= ~(size_t)3;
+    return (int)std::min<size_t>((size_t)pairs, c);
+}
+
+// pairs that X holds: a rest of three is a group of four
+static size_t adj_x_pairs(const bst_plan_s* p, int chunk) {
+    return (size_t)chunk + (p->M < 3072 && chunk % 4 == 3 ? 1 : 0);
+}
+
+// two blocks an SM over the chunk's pairs
+static int adj_fg_blocks(const bst_plan_s* p, int chunk) {
+    const int tpl = (p->M % 3 == 0) ? p->M / 12 : p->M / 16;
+    const int lpc = std::max(1, 256 / tpl);
+    return std::max(1, std::min((p->V + lpc - 1) / lpc, (304 + chunk - 1) / chunk));
 }
 
 static AdjLayout adj_layout(const bst_plan_s* p, int pairs, void* ws) {
     AdjLayout L;
     L.chunk = adj_chunk(p, pairs);
-    const size_t rows_t = (size_t)((p->N + 3) / 4) * 4;
-    float2* b = (float2*)ws;
-    L.T = b;
-    b += (size_t)L.chunk * rows_t * p->M;
+    L.fg_blocks = adj_fg_blocks(p, L.chunk);
+    // 16-byte reads of X; the workspace size has room for the rounding
+    float2* b = (float2*)(((uintptr_t)ws + 255) & ~(uintptr_t)255);
     L.X = b;
-    b += (size_t)L.chunk * p->M * p->M;
-    L.lam = b;
-    b += (size_t)L.chunk * p->V * p->M;
-    L.Y = b;
-    b += (size_t)L.chunk * p->V * p->M;
+    b += adj_x_pairs(p, L.chunk) * p->M * p->M;
+    L.T = L.lam = b;
+    b += (size_t)L.chunk * std::max(adj_rows_t(p), (size_t)p->V) * p->M;
     L.part = (float*)b;
     return L;
+}
+
+// column FFTs (stage 0) or polar stage (stage 1) of np pairs of the chunk, P to a group
+template <int M, int P>
+static void adjoint_group(bst_plan_s* p, const AdjLayout& L, int stage, int slices, int p0, int at, int np, int mode,
+                          const float* g, float* sino, bool keep_lam, cudaStream_t st) {
+    using C = AdjCfg<M>;
+    const int N = p->N, V = p->V, groups = (np + P - 1) / P;
+    float2* X = L.X + (size_t)at * M * M;
+    if (stage == 0) {
+        constexpr int LC = C::template LC<P>, CB = LC / P;
+        k_adj_col_fft<M, C::TPL, LC, P><<<dim3((M + CB - 1) / CB, groups), C::TPL * LC, C::template SC<P>, st>>>(
+            L.T + (size_t)at * adj_rows_t(p) * M, N, np, X, p->tw);
+        bst_timing_mark(p, st, 6);
+        return;
+    }
+    const Cells cl{p->cell_start, p->cell_pts, p->cell_w};
+    const float scale = (float)((double)N / (2.0 * (double)M * (double)M));
+    constexpr int LP = C::template LP<P>, LR = LP / P;
+    k_adj_polar<M, C::TPL, LP, P><<<dim3((V + LR - 1) / LR, groups), C::TPL * LP, C::template SP<P>, st>>>(
+        X, cl, V, N, slices, p0 + at, np, mode, g, (float)(2 * p->alpha), scale, sino,
+        keep_lam ? L.lam + (size_t)at * V * M : nullptr, p->tw);
+    bst_timing_mark(p, st, 7);
+}
+
+template <int M, int P>
+static bool adjoint_smem() {
+    using C = AdjCfg<M>;
+    return set_smem_a(k_adj_col_fft<M, C::TPL, C::template LC<P>, P>, C::template SC<P>) &&
+           set_smem_a(k_adj_polar<M, C::TPL, C::template LP<P>, P>, C::template SP<P>);
 }
 
 template <int M>
 static bst_status_t adjoint_chunk(bst_plan_s* p, const AdjLayout& L, const float* vol, int slices, int p0, int np,
                                   int mode, const float* g, float* sino, bool keep_lam, cudaStream_t st) {
     using C = AdjCfg<M>;
+    constexpr int PM = adj_pairs<M>();
     static std::atomic<unsigned long long> attr_done{0};
     if (!bsth::once_per_device(attr_done, [] {
-            return set_smem_a(k_adj_row_fft<M, C::TPL, C::TPC>, C::S1) &&
-                   set_smem_a(k_adj_col_fft<M, C::TPL, C::LPC>, C::S2) &&
-                   set_smem_a(k_adj_polar<M, C::TPL, C::LPC>, C::S2);
+            return set_smem_a(k_adj_row_fft<M, C::TPL, C::TPC>, C::S1) && adjoint_smem<M, 1>() &&
+                   adjoint_smem<M, 2>() && adjoint_smem<M, PM>();
         }))
         return BST_ERR_CUDA;
-    const int N = p->N, V = p->V;
-    const int row_tiles = (N + 3) / 4;
+    const int row_tiles = (p->N + 3) / 4;
     bst_timing_mark(p, st, -1);
     k_adj_row_fft<M, C::TPL, C::TPC><<<dim3((row_tiles + C::TPC - 1) / C::TPC, np), 4 * C::TPL * C::TPC, C::S1, st>>>(
-        vol, slices, p0, N, L.T, p->tw);
+        vol, slices, p0, p->N, L.T, p->tw);
     bst_timing_mark(p, st, 5);
-    k_adj_col_fft<M, C::TPL, C::LPC><<<dim3((M + C::LPC - 1) / C::LPC, np), C::TPL * C::LPC, C::S2, st>>>(
-        L.T, N, L.X, p->tw);
-    bst_timing_mark(p, st, 6);
-    Cells cl{p->cell_start, p->cell_pts, p->cell_w};
-    const float scale = (float)((double)N / (2.0 * (double)M * (double)M));
-    k_adj_polar<M, C::TPL, C::LPC><<<dim3((V + C::LPC - 1) / C::LPC, np), C::TPL * C::LPC, C::S2, st>>>(
-        L.X, cl, V, N, slices, p0, mode, g, (float)(2 * p->alpha), scale, sino, keep_lam ? L.lam : nullptr, p->tw);
-    bst_timing_mark(p, st, 7);
+    // Whole groups of PM pairs, then what remains in the smallest group that
+    // holds it.  lam overwrites T, so the polar stage starts only once every
+    // column of the chunk is transformed.
+    const int full = np / PM * PM, rem = np - full;
+    for (int stage = 0; stage < 2; ++stage) {
+        if (full > 0) adjoint_group<M, PM>(p, L, stage, slices, p0, 0, full, mode, g, sino, keep_lam, st);
+        if (rem == 1) adjoint_group<M, 1>(p, L, stage, slices, p0, full, 1, mode, g, sino, keep_lam, st);
+        if (rem == 2) adjoint_group<M, 2>(p, L, stage, slices, p0, full, 2, mode, g, sino, keep_lam, st);
+        if (rem == 3) adjoint_group<M, PM>(p, L, stage, slices, p0, full, 3, mode, g, sino, keep_lam, st);
+    }
     return BST_OK;
 }
 
@@ -407,7 +589,9 @@ static bst_status_t adjoint_chunk(bst_plan_s* p, const AdjLayout& L, const float
 
 size_t bst_adjoint_ws(const bst_plan_s* p, int slices) {
     const int pairs = (slices + 1) / 2;
-    return (size_t)bst::adj_chunk(p, pairs) * bst::adj_bytes_per_pair(p) + (size_t)pairs * p->M * sizeof(float) + 256;
+    const bst::AdjLayout L = bst::adj_layout(p, pairs, nullptr);
+    const size_t rows = (size_t)L.chunk * L.fg_blocks;
+    return (size_t)((char*)L.part - (char*)nullptr) + rows * p->M * sizeof(float) + 256;
 }
 
 bst_status_t bst_build_cells(bst_plan_s* p, cudaStream_t st) {
@@ -484,9 +668,32 @@ bst_status_t bst_launch_adjoint(bst_plan_s* p, int mode, const float* g, const f
     return cudaGetLastError() == cudaSuccess ? BST_OK : BST_ERR_CUDA;
 }
 
-// the raw ray spectrum (no weight) of pairs [p0, p0+np) into Y, from fbp.cu
-bst_status_t bst_launch_ray_spectrum(bst_plan_s* p, const float* sino, int slices, int p0, int np, float2* Y,
-                                     cudaStream_t st);
+namespace bst {
+template <int M>
+static bst_status_t launch_fg_ray_M(bst_plan_s* p, const AdjLayout& L, const float* sino, int slices, int p0, int np,
+                                    cudaStream_t st) {
+    using C = AdjCfg<M>;
+    static std::atomic<unsigned long long> attr_done{0};
+    if (!bsth::once_per_device(attr_done, [] { return set_smem_a(k_fg_ray<M, C::TPL, C::LPC>, C::SF); }))
+        return BST_ERR_CUDA;
+    bst_timing_mark(p, st, -1);
+    k_fg_ray<M, C::TPL, C::LPC><<<dim3(L.fg_blocks, np), C::TPL * C::LPC, C::SF, st>>>(
+        sino, slices, p0, p->N, p->V, L.lam, p0 > 0, L.part, p->tw);
+    bst_timing_mark(p, st, 0);
+    return BST_OK;
+}
+}  // namespace bst
+
+static bst_status_t fg_ray_dispatch(bst_plan_s* p, const bst::AdjLayout& L, const float* sino, int slices, int p0,
+                                    int np, cudaStream_t st) {
+    switch (p->M) {
+#define BST_CASE(m) \
+    case m: return bst::launch_fg_ray_M<m>(p, L, sino, slices, p0, np, st);
+        BST_FOR_EACH_M(BST_CASE)
+#undef BST_CASE
+    }
+    return BST_ERR_UNSUPPORTED_SIZE;
+}
 
 // Both gradients of <grad_vol, FBP(sino; g)>: grad_sino = the adjoint applied to
 // grad_vol (taps g; skipped when null), grad_g = sum Re(conj(lambda) Y) (skipped
@@ -497,22 +704,21 @@ bst_status_t bst_launch_backward(bst_plan_s* p, const float* sino, const float* 
     if (s != BST_OK) return s;
     const int pairs = (slices + 1) / 2;
     const bst::AdjLayout L = bst::adj_layout(p, pairs, ws);
-    const int M = p->M, V = p->V;
+    const int M = p->M;
     for (int p0 = 0; p0 < pairs; p0 += L.chunk) {
         const int np = std::min(L.chunk, pairs - p0);
         s = adjoint_chunk_dispatch(p, L, gvol, slices, p0, np, grad_sino ? BSTK_FILTER : BSTK_RAW, g, grad_sino,
                                    grad_g != nullptr, st);
         if (s != BST_OK) return s;
         if (grad_g) {
-            s = bst_launch_ray_spectrum(p, sino, slices, p0, np, L.Y, st);
+            s = fg_ray_dispatch(p, L, sino, slices, p0, np, st);
             if (s != BST_OK) return s;
-            bst::k_fg_partial<<<dim3((M + bst::FG_K - 1) / bst::FG_K, np), bst::FG_K * bst::FG_G, 0, st>>>(
-                L.lam, L.Y, V, M, p0, L.part);
         }
     }
     if (grad_g) {
         const float scale = (float)((double)p->N / (2.0 * (double)M * (double)M));
-        bst::k_fg_final<<<(M / 2 + 255) / 256, 256, 0, st>>>(L.part, pairs, M, scale, grad_g);
+        bst::k_fg_final<<<(M / 2 + bst::FG_K - 1) / bst::FG_K, bst::FG_K * bst::FG_G, 0, st>>>(
+            L.part, L.chunk * L.fg_blocks, M, scale, grad_g);
     }
     return cudaGetLastError() == cudaSuccess ? BST_OK : BST_ERR_CUDA;
 }

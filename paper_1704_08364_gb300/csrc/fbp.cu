@@ -1,8 +1,7 @@
 // fbp.cu -- plan-level entry points of the BST forward path: the plan's
 // geometry table, the dispatch of bst_fbp / bst_backproject / bst_fbp_prep on
 // the FFT length and the pad factor (the kernels are in bst_forward.cuh,
-// instantiated by fbp_pad1.cu and fbp_pad2.cu), the raw ray spectrum used by
-// the adjoint, and bst_fbp_prep.
+// instantiated by fbp_pad1.cu and fbp_pad2.cu), and bst_fbp_prep.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,9 +33,6 @@ __global__ void k_geo_table(Geo geo, int M, int* __restrict__ gJ, float2* __rest
 
 }  // namespace bst
 
-#define BST_FOR_EACH_M(X) \
-    X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048) X(4096) X(48) X(96) X(192) X(384) X(768) X(1536) X(3072)
-
 static bst_status_t forward_dispatch(bst_plan_s* p, const float* sino, int slices, int mode, const float* g,
                                      float* vol, void* ws, cudaStream_t st, int max_chunk, int lanes,
                                      const bst::PrepArgs* prep) {
@@ -63,34 +59,6 @@ bst_status_t bst_launch_forward(bst_plan_s* p, const float* sino, int slices, in
     const int chunk = std::min(pairs, p->chunk_pairs);
     const int lanes = (int)std::min<size_t>(bsth::kMaxLanes, ws_bytes / ((size_t)chunk * bsth::fwd_bytes_per_pair(p)));
     return bst_launch_forward_chunked(p, sino, slices, mode, g, vol, ws, st, p->chunk_pairs, lanes);
-}
-
-namespace bst {
-template <int M>
-bst_status_t launch_ray_spectrum_M(bst_plan_s* p, const float* sino, int slices, int p0, int np, float2* Y,
-                                   cudaStream_t st) {
-    using C = FwdCfg<M>;
-    static std::atomic<unsigned long long> attr_done{0};
-    if (!bsth::once_per_device(attr_done, [] { return set_smem(k_ray_fft<M, C::TPL, C::LPC1, 16, 0>, C::S1); }))
-        return BST_ERR_CUDA;
-    bst_timing_mark(p, st, -1);
-    k_ray_fft<M, C::TPL, C::LPC1, 16, 0><<<dim3((p->V + C::LPC1 - 1) / C::LPC1, np), C::TPL * C::LPC1, C::S1, st>>>(
-        sino, slices, p0, p->N, p->V, BSTK_RAW, nullptr, 0.f, Y, p->tw);
-    bst_timing_mark(p, st, 0);
-    return BST_OK;
-}
-}  // namespace bst
-
-// Y[pair][V][M] = unscaled DFT of the padded rays of pairs [p0, p0 + np), no weight
-bst_status_t bst_launch_ray_spectrum(bst_plan_s* p, const float* sino, int slices, int p0, int np, float2* Y,
-                                     cudaStream_t st) {
-    switch (p->M) {
-#define BST_CASE(m) \
-    case m: return bst::launch_ray_spectrum_M<m>(p, sino, slices, p0, np, Y, st);
-        BST_FOR_EACH_M(BST_CASE)
-#undef BST_CASE
-    }
-    return BST_ERR_UNSUPPORTED_SIZE;
 }
 
 bst_status_t bst_build_geo_table(bst_plan_s* p) {
