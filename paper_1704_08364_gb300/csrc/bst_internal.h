@@ -39,9 +39,9 @@ struct bst_plan_s {
     int kb_w = 0;
     float kb_poly[13] = {0};        // phi as a degree-12 polynomial in t = 2 (2x/W)^2 - 1
     float* kb_dk = nullptr;         // [N]
-    int* kb_start = nullptr;        // [kb_nstrips + 1] first work item of each strip
+    int* kb_start = nullptr;        // [kb_nstrips + 1] first item of each strip
     int* kb_list = nullptr;         // [kb_n] sample ids
-    int4* kb_items = nullptr;       // (band, first entry, end entry, 0)
+    int4* kb_items = nullptr;       // (band, first entry, end entry, 1 if the band has others)
     size_t kb_n = 0;
     int kb_nstrips = 0;
     int chunk_pairs = 1;            // slice pairs per chunk of the forward path

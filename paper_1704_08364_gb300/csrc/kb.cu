@@ -14,34 +14,53 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <new>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "bst_kb.cuh"
 
 namespace bst {
 
-template <int M, int MAXR>
-__global__ void __launch_bounds__(kb_threads<M>(), 1)
-    k_kb_col(const float2* __restrict__ Z, int V, int N, KbArgs kb, float2* __restrict__ T,
+// P slice pairs per block (blockIdx.y: group of P of the np pairs).
+// What bounds it: instruction issue (about 210 instructions a sample, item and
+// four pairs, half of them the six kernel values) and the latency of the
+// samples' loads at 16 warps an SM.  With one pair a block, strips of four columns
+// and an item a thread, every pair evaluated its own kernel values: 187 us a pair
+// at 1024 x 1024 (W = 6), 66 us with four pairs a block.
+template <int M, int MAXR, int P>
+__global__ void __launch_bounds__(kb_threads<M, P>(), kb_threads<M, P>() > 256 ? 1 : 2)
+    k_kb_col(const float2* __restrict__ Z, int np, int V, int N, KbArgs kb, float2* __restrict__ T,
              const float2* __restrict__ tw) {
     extern __shared__ float2 smem[];
-    const int pl = blockIdx.y;
+    const int pl = blockIdx.y * P;
     // strips nearest the column c' = 0 carry the most samples: start there
     const int b = blockIdx.x;
     const int strip = (b & 1) ? kb.nstrips - 1 - (b >> 1) : (b >> 1);
-    kb_col_unit<M, tpl_of<M>(), MAXR>(smem, strip, V, N, Z + (size_t)pl * V * M, kb,
-                                      T + (size_t)pl * ((N + 3) / 4) * 4 * M, tw);
+    const size_t zs = (size_t)V * M, ts = (size_t)((N + 3) / 4) * 4 * M;
+    kb_col_unit<M, tpl_of<M>(), MAXR, P>(smem, strip, min(P, np - pl), V, N, Z + pl * zs, zs, kb, T + pl * ts, ts, tw);
 }
 
-template <int M, int MAXR>
-bst_status_t launch_kb_col_M(bst_plan_s* p, const float2* Z, float2* T, int np, cudaStream_t st) {
-    constexpr size_t smem = kb_smem_bytes<M>();
+template <int M, int MAXR, int P>
+static bst_status_t launch_kb_col_P(const bst_plan_s* p, const KbArgs& a, const float2* Z, float2* T, int np,
+                                    cudaStream_t st) {
+    constexpr size_t smem = kb_smem_bytes<M, P>();
     static std::atomic<unsigned long long> attr_done{0};
     if (!bsth::once_per_device(attr_done, [] {
-            return cudaFuncSetAttribute(k_kb_col<M, MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-                   cudaSuccess;
+            return cudaFuncSetAttribute(k_kb_col<M, MAXR, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)smem) == cudaSuccess;
         }))
         return BST_ERR_CUDA;
+    k_kb_col<M, MAXR, P><<<dim3(p->kb_nstrips, (np + P - 1) / P), kb_threads<M, P>(), smem, st>>>(Z, np, p->V, p->N, a,
+                                                                                                T, p->tw);
+    return BST_OK;
+}
+
+// Whole groups of kb_pairs pairs, then what remains in the smallest group that
+// holds it.
+template <int M, int MAXR>
+bst_status_t launch_kb_col_M(bst_plan_s* p, const float2* Z, float2* T, int np, cudaStream_t st) {
     KbArgs a;
     static_assert(sizeof(a.poly) == sizeof(p->kb_poly), "polynomial size");
     for (int i = 0; i <= KB_POLY; ++i) a.poly[i] = p->kb_poly[i];
@@ -53,8 +72,14 @@ bst_status_t launch_kb_col_M(bst_plan_s* p, const float2* Z, float2* T, int np, 
     a.wq = p->wq;
     a.W = p->kb_w;
     a.nstrips = p->kb_nstrips;
-    k_kb_col<M, MAXR><<<dim3(p->kb_nstrips, np), kb_threads<M>(), smem, st>>>(Z, p->V, p->N, a, T, p->tw);
-    return BST_OK;
+    constexpr int PM = kb_pairs<M>();
+    const size_t zs = (size_t)p->V * M, ts = (size_t)((p->N + 3) / 4) * 4 * M;
+    const int full = np % PM == 3 ? np : np / PM * PM, rem = np - full;
+    bst_status_t s = BST_OK;
+    if (full > 0) s = launch_kb_col_P<M, MAXR, PM>(p, a, Z, T, full, st);
+    if (s == BST_OK && rem == 1) s = launch_kb_col_P<M, MAXR, 1>(p, a, Z + full * zs, T + full * ts, 1, st);
+    if (s == BST_OK && rem == 2) s = launch_kb_col_P<M, MAXR, 2>(p, a, Z + full * zs, T + full * ts, 2, st);
+    return s;
 }
 
 }  // namespace bst
@@ -104,14 +129,37 @@ static bool upload_vec(T** d, const std::vector<T>& h) {
     return h.empty() || cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
+// fn(begin, end) over [0, n) in up to 8 host threads; on the calling thread alone
+// where a thread cannot be started.  fn must not throw (it allocates nothing).
+template <class F>
+static void parallel(int n, F&& fn) {
+    const int most = std::min({8, n, (int)std::max(1u, std::thread::hardware_concurrency())});
+    std::vector<std::thread> t;
+    t.reserve(most);
+    int at = 0;
+    for (int i = 0; i + 1 < most; ++i) {
+        const int end = (int)((long long)n * (i + 1) / most);
+        try {
+            t.emplace_back([&fn, at, end] { fn(at, end); });
+        } catch (const std::system_error&) {
+            break;
+        }
+        at = end;
+    }
+    fn(at, n);
+    for (std::thread& x : t) x.join();
+}
+
 // Tables of KB gridding of width W for the plan, host-built in double:
 //   the kernel polynomial and the deapodization;
-//   per strip of four columns, every sample (j, k), k != 0, -M/2, whose
+//   per strip of two columns, every sample (j, k), k != 0, -M/2, whose
 //   footprint (the W columns c' - c_s in (-W/2, W/2]) meets the strip, sorted
-//   by the first row of its footprint (r' - r_s > -W/2, taken mod M);
+//   by the first row of its footprint (r' - r_s > -W/2, taken mod M), then by
+//   sample; the samples of the first KB_WMAX rows once more at the end;
 //   per band of four rows of the strip, the range of that list whose footprint
-//   meets the band (two ranges at the wrap), cut into work items of at most
-//   KB_ITEM entries; a strip's items ordered longest first.
+//   meets the band, cut into items of at most KB_ITEM entries; a strip's items
+//   ordered longest first.
+// The strips are divided over host threads.
 static bst_status_t build_kb(bst_plan_s* p, int W) {
     using bst::KB_CS;
     using bst::KB_ITEM;
@@ -174,78 +222,93 @@ static bst_status_t build_kb(bst_plan_s* p, int W) {
     }
 
     // footprint starts (first column and first row, mod M) of every sample
-    std::vector<double> cth(V), sth(V);
-    for (int j = 0; j < V; ++j) {
-        cth[j] = std::cos(p->theta[j]);
-        sth[j] = std::sin(p->theta[j]);
-    }
+    std::vector<uint16_t> fc((size_t)V * M), fr((size_t)V * M);
     auto first = [&](double x) {
         const int f = (int)std::floor(x - 0.5 * W) + 1;
-        return f < 0 ? f + M : (f >= M ? f - M : f);
+        return (uint16_t)(f < 0 ? f + M : (f >= M ? f - M : f));
     };
-    // pass 1: entries per (strip, first row)
-    std::vector<int> cnt((size_t)ns * M + 1, 0);
-    auto strips_of = [&](int fc, auto&& fn) {
-        int last = -1;
-        for (int d = 0; d < W; ++d) {
-            int c = fc + d;
-            if (c >= M) c -= M;
-            const int s = c / KB_CS;
-            if (s != last) {
-                fn(s);
-                last = s;
+    parallel(V, [&](int j0, int j1) {
+        for (int j = j0; j < j1; ++j) {
+            const double c = std::cos(p->theta[j]), s = std::sin(p->theta[j]);
+            for (int i = 0; i < M; ++i) {
+                const double k = (double)(i < M / 2 ? i : i - M);
+                fc[(size_t)j * M + i] = first(k * c);
+                fr[(size_t)j * M + i] = first(k * s);
             }
         }
-    };
-    for (int j = 0; j < V; ++j)
-        for (int kidx = 1; kidx < M; ++kidx) {
-            if (kidx == M / 2) continue;
-            const double k = (double)(kidx < M / 2 ? kidx : kidx - M);
-            const int fc = first(k * cth[j]), fr = first(k * sth[j]);
-            strips_of(fc, [&](int s) { ++cnt[(size_t)s * M + fr + 1]; });
-        }
-    for (size_t i = 0; i < (size_t)ns * M; ++i) cnt[i + 1] += cnt[i];
-    const size_t n = (size_t)cnt[(size_t)ns * M];
-    if (n >= (size_t)INT32_MAX) return BST_ERR_UNSUPPORTED_SIZE;
-    // pass 2: the lists, sorted by (strip, first row)
-    std::vector<int> list(n);
-    {
-        std::vector<int> fill(cnt.begin(), cnt.end() - 1);
+    });
+    // fn(strip, first row, sample) for the samples of strips [s0, s1), ascending by sample
+    auto each = [&](int s0, int s1, auto&& fn) {
         for (int j = 0; j < V; ++j)
-            for (int kidx = 1; kidx < M; ++kidx) {
-                if (kidx == M / 2) continue;
-                const double k = (double)(kidx < M / 2 ? kidx : kidx - M);
-                const int fc = first(k * cth[j]), fr = first(k * sth[j]);
-                strips_of(fc, [&](int s) { list[fill[(size_t)s * M + fr]++] = j * M + kidx; });
+            for (int i = 1; i < M; ++i) {
+                if (i == M / 2) continue;
+                const size_t at = (size_t)j * M + i;
+                // the strips of columns fc .. fc + W - 1 (mod M), each once
+                int s = fc[at] / KB_CS;
+                const int n = (fc[at] % KB_CS + W - 1) / KB_CS + 1;
+                for (int d = 0; d < n && d < ns; ++d, s = s + 1 == ns ? 0 : s + 1)
+                    if (s >= s0 && s < s1) fn(s, (int)fr[at], (int)at);
             }
-    }
-    // work items: band b of strip s needs first rows in [KB_RB b - W + 1, KB_RB b + KB_RB - 1] (mod M)
-    std::vector<int4> items;
-    std::vector<int> istart(ns + 1, 0);
-    auto row_pos = [&](int s, int r) { return cnt[(size_t)s * M + r]; };   // first entry with first row >= r
-    auto emit = [&](int b, int lo, int hi) {
-        for (int e = lo; e < hi; e += KB_ITEM) items.push_back(make_int4(b, e, std::min(hi, e + KB_ITEM), 0));
     };
+    // entries per (strip, first row), then the lists
+    const int wrap = std::min(bst::KB_WMAX, M);
+    std::vector<int> row((size_t)ns * (M + 1), 0);   // row[s][r]: entries of the strip with first row < r
+    std::vector<size_t> start(ns + 1, 0);            // the strip's place in the list
+    parallel(ns, [&](int s0, int s1) {
+        each(s0, s1, [&](int s, int r, int) { ++row[(size_t)s * (M + 1) + r + 1]; });
+        for (int s = s0; s < s1; ++s)
+            for (int r = 0; r < M; ++r) row[(size_t)s * (M + 1) + r + 1] += row[(size_t)s * (M + 1) + r];
+    });
     for (int s = 0; s < ns; ++s) {
-        for (int b = 0; b < nb; ++b) {
-            const int lo = KB_RB * b - W + 1, hi = KB_RB * b + KB_RB;   // rows [lo, hi)
-            if (lo >= 0) {
-                emit(b, row_pos(s, lo), row_pos(s, hi));
-            } else {
-                emit(b, row_pos(s, lo + M), row_pos(s, M));
-                emit(b, row_pos(s, 0), row_pos(s, hi));
-            }
-        }
-        // longest first: the lanes of a warp then take items of about the same
-        // length, and the block's last round of items is its shortest
-        std::stable_sort(items.begin() + istart[s], items.end(),
-                         [](const int4& a, const int4& b) { return a.z - a.y > b.z - b.y; });
-        istart[s + 1] = (int)items.size();
+        const int* q = &row[(size_t)s * (M + 1)];
+        start[s + 1] = start[s] + q[M] + q[wrap];
     }
+    const size_t n = start[ns];
+    if (n >= (size_t)INT32_MAX) return BST_ERR_UNSUPPORTED_SIZE;
+    // first entry of strip s with first row >= r, rows r >= M being those of the copy
+    auto pos = [&](int s, int r) {
+        const int* q = &row[(size_t)s * (M + 1)];
+        return (int)start[s] + (r < M ? q[r] : q[M] + q[r - M]);
+    };
+    // the entries [lo, hi) of band b of strip s: first rows [KB_RB b - W + 1, KB_RB b + KB_RB) mod M
+    auto band = [&](int s, int b) {
+        int lo = KB_RB * b - W + 1, hi = KB_RB * b + KB_RB;
+        if (lo < 0) {
+            lo += M;
+            hi += M;
+        }
+        return make_int2(pos(s, lo), pos(s, hi));
+    };
+    std::vector<int> istart(ns + 1, 0);
+    for (int s = 0; s < ns; ++s) {
+        istart[s + 1] = istart[s];
+        for (int b = 0; b < nb; ++b) {
+            const int2 e = band(s, b);
+            istart[s + 1] += (e.y - e.x + KB_ITEM - 1) / KB_ITEM;
+        }
+    }
+    std::vector<int> list(n), fill((size_t)ns * M);
+    std::vector<int4> items(istart[ns]);
+    parallel(ns, [&](int s0, int s1) {
+        for (int s = s0; s < s1; ++s)
+            for (int r = 0; r < M; ++r) fill[(size_t)s * M + r] = pos(s, r);
+        each(s0, s1, [&](int s, int r, int at) { list[fill[(size_t)s * M + r]++] = at; });
+        for (int s = s0; s < s1; ++s) {
+            const int* q = &row[(size_t)s * (M + 1)];
+            std::copy_n(list.begin() + start[s], q[wrap], list.begin() + start[s] + q[M]);
+            int4* it = items.data() + istart[s];
+            for (int b = 0; b < nb; ++b) {
+                const int2 e = band(s, b);
+                for (int i = e.x; i < e.y; i += KB_ITEM)
+                    *it++ = make_int4(b, i, std::min(e.y, i + KB_ITEM), e.y - e.x > KB_ITEM);
+            }
+            std::stable_sort(items.begin() + istart[s], items.begin() + istart[s + 1],
+                             [](const int4& a, const int4& b) { return a.z - a.y > b.z - b.y; });
+        }
+    });
 
     bst_free_kb(p);
-    bool ok = upload_vec(&p->kb_dk, dk) && upload_vec(&p->kb_start, istart) &&
-              upload_vec(&p->kb_list, list) && upload_vec(&p->kb_items, items);
+    const bool ok = upload_vec(&p->kb_dk, dk) && upload_vec(&p->kb_start, istart) && upload_vec(&p->kb_list, list) && upload_vec(&p->kb_items, items);
     if (!ok) {
         cudaGetLastError();
         bst_free_kb(p);
@@ -273,7 +336,12 @@ bst_status_t bst_plan_set_gridding(bst_plan_t p, int kind, int width) {
         return BST_ERR_INVALID_ARGUMENT;
     if (p->grid_kind == BST_GRID_KAISER_BESSEL && p->kb_w == width) return BST_OK;
     cudaDeviceSynchronize();
-    const bst_status_t s = build_kb(p, width);
+    bst_status_t s;
+    try {
+        s = build_kb(p, width);
+    } catch (const std::bad_alloc&) {
+        s = BST_ERR_OUT_OF_MEMORY;
+    }
     if (s != BST_OK) {
         p->grid_kind = BST_GRID_BILINEAR;
         return s;
