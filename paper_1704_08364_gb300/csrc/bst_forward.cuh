@@ -56,20 +56,19 @@ __global__ void __launch_bounds__(TPL * LPC, (TPL * LPC <= 1024) ? 1024 / (TPL *
                                                     two_alpha, Z + (size_t)pl * V * M, tw);
 }
 
-template <int M, int TPL, int LPC, int MAXR, int NC = 0>
+template <int M, int TPL, int LPC, int MAXR, int NC = 0, bool ILV = false>
 __global__ void __launch_bounds__(TPL * LPC, (TPL * LPC <= 1024) ? 1024 / (TPL * LPC) : 1)
     k_ray_fft_prep(const float* __restrict__ sino, int slices, int pair0, int N, int V, PrepArgs pa, int mode,
-                   const float* __restrict__ g, float two_alpha, float2* __restrict__ Z,
-                   const float2* __restrict__ tw) {
+                   float2* __restrict__ Z, const float2* __restrict__ tw) {
     extern __shared__ float2 smem[];
     const int pl = blockIdx.y;
     const int sa = 2 * (pair0 + pl), sb = sa + 1;
     const bool hb = sb < slices;
-    ray_unit_prep<M, TPL, LPC, MAXR, NC>(
+    ray_unit_prep<M, TPL, LPC, MAXR, NC, ILV>(
         smem, blockIdx.x * LPC, V, N, sino + (size_t)sa * V * N, hb ? sino + (size_t)sb * V * N : nullptr,
         pa.dark ? pa.dark + (size_t)sa * N : nullptr, (pa.dark && hb) ? pa.dark + (size_t)sb * N : nullptr,
         pa.flat ? pa.flat + (size_t)sa * N : nullptr, (pa.flat && hb) ? pa.flat + (size_t)sb * N : nullptr, pa, mode,
-        g, two_alpha, Z + (size_t)pl * V * M, tw);
+        Z + (size_t)pl * V * M, tw);
 }
 
 // gridding launches: grid (column groups, pairs), or with pair_fast

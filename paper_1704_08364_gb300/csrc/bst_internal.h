@@ -136,6 +136,12 @@ inline size_t fwd_bytes_per_pair(const bst_plan_s* p) {
     return ((size_t)p->V * p->M + rows_t * p->M) * sizeof(float2);
 }
 
+// bytes of the per-call tables of bst_fbp_prep (weight times phase of every
+// bin, window), behind the lanes of the workspace
+inline size_t prep_table_bytes(const bst_plan_s* p) {
+    return ((size_t)p->M * sizeof(float2) + (size_t)p->N * sizeof(float) + 255) & ~(size_t)255;
+}
+
 }  // namespace bsth
 
 // Record a timing mark on `st` after a launch of `stage` (or a start mark
@@ -152,9 +158,6 @@ bst_status_t bst_launch_forward_chunked(bst_plan_s* p, const float* sino, int sl
 namespace bst {
 struct PrepArgs;
 }
-// as bst_launch_forward (filter mode) with the pre-reconstruction stages in the ray kernel
-bst_status_t bst_launch_forward_prep(bst_plan_s* p, const float* sino, int slices, const bst::PrepArgs& prep,
-                                     const float* g, float* vol, void* ws, size_t ws_bytes, cudaStream_t st);
 // the forward path for pad factor 1 or 2 (fbp_pad1.cu, fbp_pad2.cu); prep may be null
 bst_status_t bst_forward_pad1(bst_plan_s* p, const float* sino, int slices, int mode, const float* g, float* vol,
                               void* ws, cudaStream_t st, int max_chunk, int lanes, const bst::PrepArgs* prep);

@@ -55,7 +55,7 @@ bst_status_t launch_forward_M(bst_plan_s* p, const float* sino, int slices, int 
     static std::atomic<unsigned long long> attr_done{0};
     if (!bsth::once_per_device(attr_done, [] {
             return set_smem(k_ray_fft<M, C::TPL, C::LPC1, MAXR, NC, C::ILV1>, C::S1) &&
-                   set_smem(k_ray_fft_prep<M, C::TPL, C::LPC1, MAXR, NC>, C::S1) &&
+                   set_smem(k_ray_fft_prep<M, C::TPL, C::LPC1, MAXR, NC, C::ILV1>, C::S1) &&
                    set_smem(k_grid_col<M, C::TPL, C::CPC, MAXR, NC>, C::S2) &&
                    set_smem(k_grid_col_paired<M, C::TPL, C::CPCP, MAXR, NC>, C::S2P) &&
                    set_smem_xchg<M, MAXR, NC>() &&
@@ -96,9 +96,9 @@ bst_status_t launch_forward_M(bst_plan_s* p, const float* sino, int slices, int 
         float2* T = Z + (size_t)chunk * V * M;
         bst_timing_mark(p, s, -1);
         if (prep)
-            k_ray_fft_prep<M, C::TPL, C::LPC1, MAXR, NC>
+            k_ray_fft_prep<M, C::TPL, C::LPC1, MAXR, NC, C::ILV1>
                 <<<dim3((V + C::LPC1 - 1) / C::LPC1, np), C::TPL * C::LPC1, C::S1, s>>>(
-                    sino, slices, p0, N, V, *prep, mode, g, two_alpha, Z, p->tw);
+                    sino, slices, p0, N, V, *prep, mode, Z, p->tw);
         else
             k_ray_fft<M, C::TPL, C::LPC1, MAXR, NC, C::ILV1><<<dim3((V + C::LPC1 - 1) / C::LPC1, np), C::TPL * C::LPC1, C::S1, s>>>(
                 sino, slices, p0, N, V, mode, g, two_alpha, Z, p->tw);

@@ -82,6 +82,20 @@ __device__ __forceinline__ void spec_store(float2* z, int j, int V, int M, int m
     }
 }
 
+// Weight W[|k|] of bin k for `mode` (times the polar cell area |k|, 1/4 at
+// k = 0, with BSTK_KBW); the Nyquist bin is zero unless the mode is raw.
+__device__ __forceinline__ float bin_weight(int k, int M, int mode, const float* __restrict__ g, float two_alpha) {
+    const int ak = k <= (M >> 1) ? k : M - k;
+    const int md = mode & 7;
+    float w;
+    if (md == BSTK_RAW) w = 1.f;
+    else if (ak == (M >> 1)) w = 0.f;
+    else if (md == BSTK_FILTER) w = g ? __ldg(g + ak) : 1.f;
+    else w = ak == 0 ? 0.f : __fdiv_rn(two_alpha, (float)ak);
+    if (mode & BSTK_KBW) w *= ak == 0 ? 0.25f : (float)ak;
+    return w;
+}
+
 struct SpecDst {
     float2* z;      // the pair's spectrum
     int j, V;       // row (angle) of this line, rows of the pair
@@ -92,14 +106,7 @@ struct SpecDst {
     static constexpr bool kSmem = false;
     __device__ __forceinline__ void store(int k, float2 v) const {
         if (!live) return;
-        const int ak = k <= (M >> 1) ? k : M - k;
-        const int md = mode & 7;
-        float w;
-        if (md == BSTK_RAW) w = 1.f;
-        else if (ak == (M >> 1)) w = 0.f;
-        else if (md == BSTK_FILTER) w = g ? __ldg(g + ak) : 1.f;
-        else w = ak == 0 ? 0.f : __fdiv_rn(two_alpha, (float)ak);
-        if (mode & BSTK_KBW) w *= ak == 0 ? 0.25f : (float)ak;
+        const float w = bin_weight(k, M, mode, g, two_alpha);
         spec_store(z, j, V, M, mode, k, make_float2(v.x * w, v.y * w));
     }
 };
@@ -283,111 +290,99 @@ template <int M> __host__ __device__ constexpr int row_line_stride() { return sm
 // Window (stage P1): y_i *= w(t_i - shift dt), a Kaiser-Bessel window
 // I0(b sqrt(1 - (t/h)^2)) / I0(b) for |t| <= h.  Centering (Sec. 1 (b)): the
 // spectrum is multiplied by exp(+2 pi i k shift / M), the exact shift of the
-// padded ray by `shift` samples.
+// padded ray by `shift` samples.  The window and the weight times the phase
+// depend on the sample and the bin only: a small kernel (k_prep_tables) fills
+// two tables per call, and the ray kernel reads them.  Evaluating them per
+// output (a 64-bit modulo, two sincospif; I0 per sample) made the ray kernel
+// issue 65.0 M warp instructions a pair at 2048 x 2000 against 22.9 M without
+// the stages: 95.7 us a pair, 66.9 us with the tables, 50 us
+// with the rays requested before the first is used (prep_gather).
 struct PrepArgs {
     const float* dark;    // [S][N] or null (0)
     const float* flat;    // [S][N] or null (input is already y)
-    float shift;          // centering shift in detector samples
-    int shift_int;        // its integer part ...
-    float shift_frac;     // ... and fraction (exact phase reduction)
-    float kb_beta;        // window shape (0: no window)
-    float kb_inv_half;    // 1 / half-width (detector units)
-    float kb_norm;        // 1 / I0(kb_beta)
+    const float* win;     // [N] window, or null
+    const float2* cw;     // [M] weight times phase of every bin
 };
 
-template <int NC = 0>
-struct RaySrcPrep {
+// One angle's rays of a slice pair and the rows that prepare them.
+struct PrepRays {
     const float* ya;
-    const float* yb;
+    const float* yb;    // or null
     const float* da;
     const float* db;
     const float* fa;
     const float* fb;
-    int N, M;
-    bool live;
-    PrepArgs pa;
-    static constexpr bool kSmem = false;
-    static __host__ __device__ constexpr bool zero_group(int lo, int hi, int Mc) {
-        return NC > 0 && lo >= NC / 2 && hi <= Mc - NC / 2;
-    }
-    __device__ __forceinline__ float sample(const float* y, const float* d, const float* f, int i) const {
-        float v = __ldg(y + i);
-        if (f) {
-            const float dk = d ? __ldg(d + i) : 0.f;
-            v = -logf(fmaxf(v - dk, 1e-6f) / fmaxf(__ldg(f + i) - dk, 1e-6f));
-        }
-        return v;
-    }
-    __device__ __forceinline__ float2 load(int m) const {
-        const int n = NC > 0 ? NC : N;
-        int i = m + (n >> 1);
-        if (i >= M) i -= M;
-        if (!live || i >= n) return make_float2(0.f, 0.f);
-        float w = 1.f;
-        if (pa.kb_beta > 0.f) {
-            const float t = ((float)(i - (n >> 1)) - pa.shift) * (2.f / (float)n);
-            const float u = t * pa.kb_inv_half;
-            w = fabsf(u) <= 1.f ? cyl_bessel_i0f(pa.kb_beta * sqrtf(fmaxf(1.f - u * u, 0.f))) * pa.kb_norm : 0.f;
-        }
-        return make_float2(w * sample(ya, da, fa, i), yb ? w * sample(yb, db, fb, i) : 0.f);
+    const float* win;
+    __device__ __forceinline__ static float sample(float v, const float* d, const float* f, int i) {
+        if (!f) return v;
+        const float dk = d ? __ldg(d + i) : 0.f;
+        return -logf(fmaxf(v - dk, 1e-6f) / fmaxf(__ldg(f + i) - dk, 1e-6f));
     }
 };
 
-struct SpecDstShift {
+// The prepared first-pass inputs x[i] = padded ray at t + i TPL of one line, for
+// fft_line_regs: all rays are requested before the first is used (their latency
+// bounds the kernel, and the logarithms between two loads would hold the next
+// one back).  live: the line exists; n: ray count (NC if known).
+template <int M, int TPL, int NC>
+__device__ __forceinline__ void prep_gather(const PrepRays& r, int t, int N, bool live, float2 (&x)[M / TPL]) {
+    const int n = NC > 0 ? NC : N, h = n >> 1;
+#pragma unroll
+    for (int i = 0; i < M / TPL; ++i) {
+        x[i] = make_float2(0.f, 0.f);
+        if (NC > 0 && i * TPL >= NC / 2 && (i + 1) * TPL <= M - NC / 2) continue;   // padding
+        int m = t + i * TPL + h;
+        if (m >= M) m -= M;
+        if (live && m < n) x[i] = make_float2(__ldg(r.ya + m), r.yb ? __ldg(r.yb + m) : 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < M / TPL; ++i) {
+        if (NC > 0 && i * TPL >= NC / 2 && (i + 1) * TPL <= M - NC / 2) continue;
+        int m = t + i * TPL + h;
+        if (m >= M) m -= M;
+        if (live && m < n) {
+            const float w = r.win ? __ldg(r.win + m) : 1.f;
+            x[i] = make_float2(w * PrepRays::sample(x[i].x, r.da, r.fa, m),
+                               r.yb ? w * PrepRays::sample(x[i].y, r.db, r.fb, m) : 0.f);
+        }
+    }
+}
+
+struct SpecDstPrep {
     float2* z;      // the pair's spectrum
     int j, V;       // row (angle) of this line, rows of the pair
-    const float* g;
+    const float2* cw;
     int M, mode;
-    float two_alpha;
     bool live;
-    PrepArgs pa;
     static constexpr bool kSmem = false;
     __device__ __forceinline__ void store(int k, float2 v) const {
-        if (!live) return;
-        const int ak = k <= (M >> 1) ? k : M - k;
-        const int md = mode & 7;
-        float w;
-        if (ak == (M >> 1)) w = 0.f;
-        else if (md == BSTK_FILTER) w = g ? __ldg(g + ak) : 1.f;
-        else w = ak == 0 ? 0.f : __fdiv_rn(two_alpha, (float)ak);
-        if (mode & BSTK_KBW) w *= ak == 0 ? 0.25f : (float)ak;
-        if (pa.shift != 0.f) {
-            // exp(+2 pi i k s / M) with s = s_int + s_frac; the integer part reduced exactly mod M
-            const int ks = signed_freq(k, M);
-            int m = (int)(((long long)ks * pa.shift_int) % M);
-            if (m < 0) m += M;
-            float s1, c1, s2, c2;
-            sincospif(2.f * (float)m / (float)M, &s1, &c1);
-            sincospif(2.f * (float)ks * pa.shift_frac / (float)M, &s2, &c2);
-            const float c = c1 * c2 - s1 * s2, sn = s1 * c2 + c1 * s2;
-            v = make_float2(v.x * c - v.y * sn, v.x * sn + v.y * c);
-        }
-        spec_store(z, j, V, M, mode, k, make_float2(v.x * w, v.y * w));
+        if (live) spec_store(z, j, V, M, mode, k, cmul(v, __ldg(cw + k)));
     }
 };
-
-// ray_unit with the pre-reconstruction stages (slice rows da/db, fa/fb of the
-// dark and flat fields, or null)
-template <int M, int TPL, int LPC, int MAXR, int NC = 0>
-__device__ __forceinline__ void ray_unit_prep(float2* smem, int j0, int V, int N, const float* __restrict__ ya,
-                                              const float* __restrict__ yb, const float* da, const float* db,
-                                              const float* fa, const float* fb, const PrepArgs& pa, int mode,
-                                              const float* __restrict__ g, float two_alpha,
-                                              float2* __restrict__ Zp, const float2* __restrict__ tw) {
-    const int line = threadIdx.x / TPL, t = threadIdx.x % TPL;
-    const int j = j0 + line;
-    const bool live = j < V;
-    const int jj = live ? j : 0;
-    RaySrcPrep<NC> src{ya + (size_t)jj * N, yb ? yb + (size_t)jj * N : nullptr, da, db, fa, fb, N, M, live, pa};
-    SpecDstShift dst{Zp, jj, V, g, M, mode, two_alpha, live, pa};
-    SmemLine sm{smem + line * smem_line_len(M)};
-    fft_line<M, TPL, false, MAXR>(t, src, dst, sm, tw);
-}
 
 // Shared-memory stride between the lines of a ray unit: with the lines
 // interleaved over the lanes (ILV), the lines are skewed by 16 banks so that
 // lanes of two lines at the same offset do not share a bank.
 template <int M, bool ILV> __host__ __device__ constexpr int ray_line_stride() { return smem_line_len(M) + (ILV ? 8 : 0); }
+
+// ray_unit with the pre-reconstruction stages (slice rows da/db, fa/fb of the
+// dark and flat fields, or null)
+template <int M, int TPL, int LPC, int MAXR, int NC = 0, bool ILV = false>
+__device__ __forceinline__ void ray_unit_prep(float2* smem, int j0, int V, int N, const float* __restrict__ ya,
+                                              const float* __restrict__ yb, const float* da, const float* db,
+                                              const float* fa, const float* fb, const PrepArgs& pa, int mode,
+                                              float2* __restrict__ Zp, const float2* __restrict__ tw) {
+    const int line = ILV ? threadIdx.x % LPC : threadIdx.x / TPL, t = ILV ? threadIdx.x / LPC : threadIdx.x % TPL;
+    const int j = j0 + line;
+    const bool live = j < V;
+    const int jj = live ? j : 0;
+    const PrepRays rays{ya + (size_t)jj * N, yb ? yb + (size_t)jj * N : nullptr, da, db, fa, fb, pa.win};
+    const SpecDstPrep dst{Zp, jj, V, pa.cw, M, mode, live};
+    const SmemLine sm{smem + line * ray_line_stride<M, ILV>()};
+    float2 x[M / TPL];
+    prep_gather<M, TPL, NC>(rays, t, N, live, x);
+    fft_line_regs<M, TPL, false, MAXR, SpecDstPrep, BlockSync, true>(t, x, dst, sm, tw);
+}
 
 // P2 + P3 + P4 for lines j0 .. j0 + LPC - 1 of one slice pair (TPL * LPC
 // threads; tid the thread's index among them, -1: threadIdx.x; `sync` the

@@ -31,6 +31,27 @@ __global__ void k_geo_table(Geo geo, int M, int* __restrict__ gJ, float2* __rest
     gF[idx] = f;
 }
 
+// The tables of the pre-reconstruction stages: cw[k] = weight(k) exp(+2 pi i k
+// shift / M) and, with win, the window at the measured samples (evaluated in
+// double; which samples lie inside it is decided in float).
+__global__ void k_prep_tables(int M, int N, int mode, const float* __restrict__ g, float two_alpha, float shift,
+                              float beta, float half, float2* __restrict__ cw, float* __restrict__ win) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < M) {
+        double s, c;
+        sincospi(2.0 * (double)signed_freq(i, M) * (double)shift / (double)M, &s, &c);
+        const double w = (double)bin_weight(i, M, mode, g, two_alpha);
+        cw[i] = make_float2((float)(w * c), (float)(w * s));
+    }
+    if (win && i < N) {
+        const float uf = ((float)(i - (N >> 1)) - shift) * (2.f / (float)N) * (1.f / half);
+        const double u = ((double)(i - (N >> 1)) - (double)shift) * (2.0 / (double)N) / (double)half;
+        win[i] = fabsf(uf) <= 1.f ? (float)(cyl_bessel_i0((double)beta * sqrt(fmax(1.0 - u * u, 0.0))) /
+                                            cyl_bessel_i0((double)beta))
+                                  : 0.f;
+    }
+}
+
 }  // namespace bst
 
 static bst_status_t forward_dispatch(bst_plan_s* p, const float* sino, int slices, int mode, const float* g,
@@ -43,14 +64,6 @@ static bst_status_t forward_dispatch(bst_plan_s* p, const float* sino, int slice
 bst_status_t bst_launch_forward_chunked(bst_plan_s* p, const float* sino, int slices, int mode, const float* g,
                                         float* vol, void* ws, cudaStream_t st, int max_chunk, int lanes) {
     return forward_dispatch(p, sino, slices, mode, g, vol, ws, st, max_chunk, lanes, nullptr);
-}
-
-bst_status_t bst_launch_forward_prep(bst_plan_s* p, const float* sino, int slices, const bst::PrepArgs& prep,
-                                     const float* g, float* vol, void* ws, size_t ws_bytes, cudaStream_t st) {
-    const int pairs = (slices + 1) / 2;
-    const int chunk = std::min(pairs, p->chunk_pairs);
-    const int lanes = (int)std::min<size_t>(bsth::kMaxLanes, ws_bytes / ((size_t)chunk * bsth::fwd_bytes_per_pair(p)));
-    return forward_dispatch(p, sino, slices, BSTK_FILTER, g, vol, ws, st, p->chunk_pairs, lanes, &prep);
 }
 
 bst_status_t bst_launch_forward(bst_plan_s* p, const float* sino, int slices, int mode, const float* g, float* vol,
@@ -84,14 +97,16 @@ extern "C" bst_status_t bst_fbp_prep(bst_plan_t p, const float* d_sino, int slic
     const uintptr_t a0 = (uintptr_t)d_sino, b0 = (uintptr_t)d_volume;
     if (a0 < b0 + nv && b0 < a0 + ns) return BST_ERR_INVALID_ARGUMENT;
     if (!d_ws || ws_bytes < bst_workspace_bytes(p, slices)) return BST_ERR_WORKSPACE_TOO_SMALL;
-    bst::PrepArgs pa;
-    pa.dark = d_dark;
-    pa.flat = d_flat;
-    pa.shift = shift;
-    pa.shift_int = (int)std::floor(shift);
-    pa.shift_frac = (float)((double)shift - std::floor((double)shift));
-    pa.kb_beta = kb_beta;
-    pa.kb_inv_half = kb_beta > 0.f ? 1.f / kb_halfwidth : 0.f;
-    pa.kb_norm = kb_beta > 0.f ? (float)(1.0 / bst_bessel_i0((double)kb_beta)) : 1.f;
-    return bst_launch_forward_prep(p, d_sino, slices, pa, d_g, d_volume, d_ws, ws_bytes, (cudaStream_t)stream);
+    const int chunk = std::min((slices + 1) / 2, p->chunk_pairs);
+    const size_t lane = (size_t)chunk * bsth::fwd_bytes_per_pair(p);
+    const int lanes = (int)std::min<size_t>(bsth::kMaxLanes, (ws_bytes - bsth::prep_table_bytes(p)) / lane);
+    float2* cw = (float2*)((char*)d_ws + lanes * lane);
+    float* win = kb_beta > 0.f ? (float*)(cw + p->M) : nullptr;
+    const cudaStream_t st = (cudaStream_t)stream;
+    bst::k_prep_tables<<<(std::max(p->M, p->N) + 127) / 128, 128, 0, st>>>(
+        p->M, p->N, BSTK_FILTER | (p->grid_kind == BST_GRID_KAISER_BESSEL ? BSTK_KBW : 0), d_g, (float)(2 * p->alpha),
+        shift, kb_beta, kb_halfwidth, cw, win);
+    const bst::PrepArgs pa{d_dark, d_flat, win, cw};
+    return forward_dispatch(p, d_sino, slices, BSTK_FILTER, d_g, d_volume, d_ws, st, p->chunk_pairs, lanes, &pa);
 }
+

@@ -243,7 +243,7 @@ size_t bst_workspace_bytes(bst_plan_t p, int slices) {
     const int chunk = std::min(pairs, p->chunk_pairs);
     const int nchunks = (pairs + chunk - 1) / chunk;
     const int lanes = std::min(std::min(nchunks, bsth::kMaxLanes), std::max(p->max_lanes, 1));   // chunks in flight
-    return (size_t)lanes * chunk * bsth::fwd_bytes_per_pair(p);
+    return (size_t)lanes * chunk * bsth::fwd_bytes_per_pair(p) + bsth::prep_table_bytes(p);
 }
 
 size_t bst_adjoint_workspace_bytes(bst_plan_t p, int slices) {
