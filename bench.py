@@ -104,7 +104,8 @@ STAGE_NAMES = {0: "k_ray_fft", 1: "k_grid_col", 2: "k_row_ifft", 3: "k_ss_filter
 # to its `sha` and the benchmark runs the same shape; otherwise the roofline
 # reports traffic null.
 KERNEL_SOURCES = ["paper_1704_08364_gb300/csrc/bst_forward.cuh", "paper_1704_08364_gb300/csrc/bst_stages.cuh",
-                  "paper_1704_08364_gb300/csrc/bst_fft.cuh", "paper_1704_08364_gb300/csrc/bst_geo.cuh"]
+                  "paper_1704_08364_gb300/csrc/bst_fft.cuh", "paper_1704_08364_gb300/csrc/bst_geo.cuh",
+                  "paper_1704_08364_gb300/csrc/bst_inter.cuh"]
 CAPTURED_TRAFFIC = [
     {"sha": "5182a6ef3146a9c4f464342e17da68624378eacd4d1d37d661da52193c60e7df",
      "rays": 2048, "pad": 2,

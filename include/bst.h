@@ -70,8 +70,11 @@ typedef enum {
  * (an implementation choice; the paper's stages P3-P5 fix the values only). */
 typedef enum {
     BST_LAYOUT_PACKED = 0,  /* Z[V][M] complex64, natural order of k */
-    BST_LAYOUT_PAIRED = 1   /* Z[V][M/2] pairs (Z[k], Z[-k]): one 16-byte load serves a
+    BST_LAYOUT_PAIRED = 1,  /* Z[V][M/2] pairs (Z[k], Z[-k]): one 16-byte load serves a
                                Cartesian point and its mirror (bilinear gridding only) */
+    BST_LAYOUT_INTERLEAVED = 2  /* groups of 2 to 8 slice pairs interleaved point by point
+                               (FFT lengths from 32); pairs that fill no group take the
+                               paired layout */
 } bst_layout_t;
 
 /* Launch shape of the forward path (extension; no passage: the paper fixes
@@ -80,7 +83,8 @@ typedef enum {
 typedef struct {
     int max_radix;    /* largest Stockham radix: 16 or 8 */
     int layout;       /* bst_layout_t */
-    int chunk_pairs;  /* slice pairs per launch of each stage, 1..256 */
+    int chunk_pairs;  /* slice pairs per launch of each stage at most, 1..256 (a call that
+                         fits in one chunk may be split over the lanes) */
     int pair_fast;    /* 1: gridding blocks ordered pair-fastest within a chunk */
     int max_lanes;    /* streams alternating chunks, 1 or 2 */
     int grid_xchg;    /* paired layout only: 1 feeds the first column-FFT pass of both
@@ -300,18 +304,19 @@ bst_status_t bst_plan_get_gridding(bst_plan_t plan, int* kind, int* width);
  * layout a bst_layout_t, chunk_pairs 1..256, pair_fast 0 or 1, max_lanes 1
  * or 2) and changes nothing on error; bst_workspace_bytes follows the new
  * chunk and lane counts, so size workspaces after setting it.  A plan starts
- * with radix 16, the packed layout, chunks sized to about 64 MiB of
- * workspace, block order column-fastest and two lanes.  A Kaiser-Bessel plan
+ * with radix 16, the interleaved layout, grid_xchg 1, chunks of about 64 MiB of
+ * workspace but at least 8 pairs, block order pair-fastest from M = 2048 on,
+ * and two lanes.  A workspace that is not 16-byte aligned takes the packed
+ * layout whatever the field says.  A Kaiser-Bessel plan
  * always uses the packed layout.  Errors: INVALID_ARGUMENT. */
 bst_status_t bst_plan_set_forward_config(bst_plan_t plan, const bst_fwd_config_t* config);
 bst_status_t bst_plan_get_forward_config(bst_plan_t plan, bst_fwd_config_t* config);
 
 /* Autotuner (extension; no passage): time the plan's forward path on a
- * synthetic batch of about 256 MiB (`slices` slices, at least 4, and at
- * least 64 where the default chunk is one pair; <= 0 picks that size) under
- * each candidate launch shape -- radix 16 or 8; packed or
- * paired layout (bilinear plans); the plan's default chunk and, where that
- * is one pair, chunks of 2, 4 and 8 pairs; either block order -- keep the fastest
+ * synthetic batch of about 256 MiB (`slices` slices, at least two chunks of the
+ * largest candidate; <= 0 picks that size) under each candidate launch shape --
+ * radix 16 or 8; interleaved or paired layout (bilinear plans); half the plan's
+ * default chunk, the default and twice it; either block order -- keep the fastest
  * (the best of three timed runs each, after one warm-up run) and return its
  * radix in *chosen (may be NULL).  Allocates and frees its own buffers;
  * synchronises the device. */

@@ -18,6 +18,7 @@ FILTER = 0
 BACKPROJECT = 1
 GRID_BILINEAR = 0
 GRID_KAISER_BESSEL = 1
+_LAYOUTS = ("packed", "paired", "interleaved")   # bst_layout_t
 
 
 class BstError(RuntimeError):
@@ -112,11 +113,11 @@ class Plan:
     @property
     def forward_config(self) -> dict:
         """Launch shape of the forward path (bst_plan_get_forward_config):
-        max_radix, layout ("packed" or "paired"), chunk_pairs, pair_fast, max_lanes,
+        max_radix, layout ("packed", "paired" or "interleaved"), chunk_pairs, pair_fast, max_lanes,
         grid_xchg (1: register-fed paired gridding, 0: through shared memory)."""
         c = _lib.FwdConfig()
         _check(self._lib.bst_plan_get_forward_config(self._h, ctypes.byref(c)), "bst_plan_get_forward_config")
-        return {"max_radix": c.max_radix, "layout": "paired" if c.layout == 1 else "packed",
+        return {"max_radix": c.max_radix, "layout": _LAYOUTS[c.layout],
                 "chunk_pairs": c.chunk_pairs, "pair_fast": c.pair_fast, "max_lanes": c.max_lanes,
                 "grid_xchg": c.grid_xchg}
 
@@ -125,7 +126,7 @@ class Plan:
         results are identical up to rounding whatever the shape."""
         cur = self.forward_config
         cur.update(kw)
-        layout = {"packed": 0, "paired": 1}.get(cur["layout"], cur["layout"])
+        layout = _LAYOUTS.index(cur["layout"]) if cur["layout"] in _LAYOUTS else cur["layout"]
         c = _lib.FwdConfig(int(cur["max_radix"]), int(layout),
                            int(cur["chunk_pairs"]), int(cur["pair_fast"]), int(cur["max_lanes"]),
                            int(cur["grid_xchg"]))

@@ -3,8 +3,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
-
 #include <vector>
 
 #include "../../include/bst.h"
@@ -134,6 +134,27 @@ inline bool check_cuda(cudaError_t e) { return e == cudaSuccess; }
 inline size_t fwd_bytes_per_pair(const bst_plan_s* p) {
     const size_t rows_t = (size_t)((p->N + 3) / 4) * 4;
     return ((size_t)p->V * p->M + rows_t * p->M) * sizeof(float2);
+}
+
+// Slice pairs of a group of the interleaved layout for FFT length M (1: the
+// length has none): 256 / (threads per line), at most 8 and a multiple of the
+// rows that a half-warp covers (bst_inter.cuh).
+__host__ __device__ constexpr int inter_pairs_of(int M) {
+    const int tpl = M % 3 == 0 ? M / 12 : M / 16;
+    const int c = 256 / tpl > 8 ? 8 : tpl >= 256 ? 2 : 256 / tpl;
+    return c > 0 && tpl % (16 / c) == 0 ? c : 1;
+}
+
+// Slice pairs per chunk for a call of `pairs` pairs with at most `most` a chunk.
+// A call that would be one chunk is split over the two lanes, in whole groups,
+// where the halves still fill the GPU: one half's gridding then overlaps the
+// other's FFTs.  The line, pairs M^2 >= 2^23, is a call of about 80 us: below it a
+// half's kernels are shorter than their launches.
+inline int fwd_chunk(const bst_plan_s* p, int pairs, int most) {
+    const int c = std::min(pairs, most);
+    if (p->max_lanes < 2 || c < pairs || pairs < 2 || (long long)pairs * p->M * p->M < (1ll << 23)) return c;
+    const int g = inter_pairs_of(p->M), h = (pairs + 1) / 2;
+    return std::min(pairs, (h + g - 1) / g * g);
 }
 
 // bytes of the per-call tables of bst_fbp_prep (weight times phase of every

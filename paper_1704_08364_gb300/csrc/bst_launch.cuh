@@ -7,8 +7,10 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cstdint>
 
 #include "bst_forward.cuh"
+#include "bst_inter.cuh"
 
 namespace bst {
 
@@ -48,6 +50,24 @@ static bool set_smem_xchg() {
     return true;
 }
 
+// shared memory of the interleaved kernels, and their opt-in, for the lengths
+// that have them
+template <int M> struct InterCfg {
+    static constexpr int P = inter_pairs<M>(), LP = inter_lanes<P>(), TPL = tpl_of<M>();
+    static constexpr bool OK = P > 1;
+    static constexpr size_t S1 = (size_t)inter_ray_rows<M>() * LP * inter_stride<M>(LP) * sizeof(float2);
+    static constexpr size_t S2 = (size_t)2 * P * inter_stride<M>(P) * sizeof(float2);
+    static constexpr size_t S3 = (size_t)4 * inter_row_tiles<M>() * row_line_stride<M>() * sizeof(float2);
+};
+template <int M, int MAXR, int NC>
+static bool set_smem_inter() {
+    using I = InterCfg<M>;
+    if constexpr (I::OK)
+        return set_smem(k_ray_inter<M, MAXR, NC, false>, I::S1) && set_smem(k_ray_inter<M, MAXR, NC, true>, I::S1) &&
+               set_smem(k_grid_inter<M, MAXR, NC>, I::S2) && set_smem(k_row_inter<M, MAXR, NC>, I::S3);
+    return true;
+}
+
 template <int M, int MAXR, int NC>
 bst_status_t launch_forward_M(bst_plan_s* p, const float* sino, int slices, int mode, const float* g, float* vol,
                               void* ws, cudaStream_t st, int max_chunk, int lanes, const PrepArgs* prep) {
@@ -58,13 +78,13 @@ bst_status_t launch_forward_M(bst_plan_s* p, const float* sino, int slices, int 
                    set_smem(k_ray_fft_prep<M, C::TPL, C::LPC1, MAXR, NC, C::ILV1>, C::S1) &&
                    set_smem(k_grid_col<M, C::TPL, C::CPC, MAXR, NC>, C::S2) &&
                    set_smem(k_grid_col_paired<M, C::TPL, C::CPCP, MAXR, NC>, C::S2P) &&
-                   set_smem_xchg<M, MAXR, NC>() &&
+                   set_smem_xchg<M, MAXR, NC>() && set_smem_inter<M, MAXR, NC>() &&
                    set_smem(k_row_ifft<M, C::TPL, C::TPC, MAXR, NC>, C::S3);
         }))
         return BST_ERR_CUDA;
     const int N = p->N, V = p->V;
     const int pairs = (slices + 1) / 2;
-    const int chunk = std::min(pairs, max_chunk);
+    const int chunk = lanes > 1 ? bsth::fwd_chunk(p, pairs, max_chunk) : std::min(pairs, max_chunk);
     const int nchunks = (pairs + chunk - 1) / chunk;
     // chunks rotate over up to kMaxLanes streams (each with its own part of the
     // workspace) so that one chunk's gridding overlaps the next chunk's FFTs;
@@ -77,8 +97,14 @@ bst_status_t launch_forward_M(bst_plan_s* p, const float* sino, int slices, int 
     const int row_tiles = (N + 3) / 4;
     const bool kbg = p->grid_kind == BST_GRID_KAISER_BESSEL;
     if (kbg && mode != BSTK_RAW) mode |= BSTK_KBW;
-    // the paired spectrum layout serves the bilinear gridding kernel only
-    const bool paired = !kbg && mode != BSTK_RAW && p->fwd_layout == BST_LAYOUT_PAIRED;
+    // The paired and interleaved layouts serve the bilinear gridding only; their
+    // kernels read the workspace 16 bytes at a time, so a workspace that is not
+    // so aligned takes the packed layout.  Groups of inter_pairs<M>() slice
+    // pairs are interleaved; what remains of a chunk is paired.
+    const bool wide = !kbg && mode != BSTK_RAW && ((uintptr_t)ws & 15) == 0;
+    const bool paired = wide && p->fwd_layout != BST_LAYOUT_PACKED;
+    const bool inter = wide && p->fwd_layout == BST_LAYOUT_INTERLEAVED && InterCfg<M>::OK;
+    const int base_mode = mode;
     if (paired) mode |= BSTK_PAIRED;
     const int pf = p->pair_fast ? 1 : 0;
     const float* dk = kbg ? p->kb_dk : nullptr;
@@ -87,13 +113,30 @@ bst_status_t launch_forward_M(bst_plan_s* p, const float* sino, int slices, int 
         for (int l = 0; l < nl; ++l)
             if (cudaStreamWaitEvent(p->lane[l], p->ev_fork, 0) != cudaSuccess) return BST_ERR_CUDA;
     }
-    for (int c = 0; c < nchunks; ++c) {
-        const int p0 = c * chunk;
-        const int np = std::min(chunk, pairs - p0);
-        const int l = c % nl;
-        cudaStream_t s = nl > 1 ? p->lane[l] : st;
-        float2* Z = (float2*)ws + (size_t)l * lane_elems;
-        float2* T = Z + (size_t)chunk * V * M;
+    // the three stages of np pairs from pair p0 on stream s, groups interleaved
+    auto run_inter = [&](int p0, int np, float2* Z, float2* T, cudaStream_t s) {
+        if constexpr (InterCfg<M>::OK) {
+            using I = InterCfg<M>;
+            constexpr int RJ = inter_ray_rows<M>(), RT = inter_row_tiles<M>() * (4 / I::LP);
+            const dim3 gr((V + RJ - 1) / RJ, np / I::LP), gc(np / I::P, M / 2);
+            bst_timing_mark(p, s, -1);
+            if (prep)
+                k_ray_inter<M, MAXR, NC, true><<<gr, inter_ray_threads<M>(), I::S1, s>>>(
+                    sino, slices, p0, N, V, *prep, base_mode, g, two_alpha, Z, p->tw);
+            else
+                k_ray_inter<M, MAXR, NC, false><<<gr, inter_ray_threads<M>(), I::S1, s>>>(
+                    sino, slices, p0, N, V, PrepArgs{}, base_mode, g, two_alpha, Z, p->tw);
+            bst_timing_mark(p, s, 0);
+            k_grid_inter<M, MAXR, NC><<<pf ? gc : dim3(gc.y, gc.x), 2 * I::P * I::TPL, I::S2, s>>>(
+                Z, V, N, p->geo_J, p->geo_f, T, p->tw, pf);
+            bst_timing_mark(p, s, 1);
+            k_row_inter<M, MAXR, NC><<<dim3((N + RT - 1) / RT, np / I::LP), 4 * I::TPL * inter_row_tiles<M>(), I::S3, s>>>(
+                T, slices, p0, N, scale, vol, p->tw);
+            bst_timing_mark(p, s, 2);
+        }
+    };
+    // ... packed or paired
+    auto run_pairs = [&](int p0, int np, float2* Z, float2* T, cudaStream_t s) {
         bst_timing_mark(p, s, -1);
         if (prep)
             k_ray_fft_prep<M, C::TPL, C::LPC1, MAXR, NC, C::ILV1>
@@ -125,6 +168,22 @@ bst_status_t launch_forward_M(bst_plan_s* p, const float* sino, int slices, int 
         k_row_ifft<M, C::TPL, C::TPC, MAXR, NC><<<dim3((row_tiles + C::TPC - 1) / C::TPC, np), 4 * C::TPL * C::TPC, C::S3, s>>>(
             T, slices, p0, N, scale, vol, p->tw, dk);
         bst_timing_mark(p, s, 2);
+        return BST_OK;
+    };
+    for (int c = 0; c < nchunks; ++c) {
+        const int p0 = c * chunk;
+        const int np = std::min(chunk, pairs - p0);
+        const int l = c % nl;
+        cudaStream_t s = nl > 1 ? p->lane[l] : st;
+        float2* Z = (float2*)ws + (size_t)l * lane_elems;
+        float2* T = Z + (size_t)chunk * V * M;
+        const int ni = inter ? np / InterCfg<M>::P * InterCfg<M>::P : 0;
+        if (ni > 0) run_inter(p0, ni, Z, T, s);
+        if (ni < np) {
+            const bst_status_t rs = run_pairs(p0 + ni, np - ni, Z + (size_t)ni * V * M,
+                                              T + (size_t)ni * ((N + 3) / 4) * 4 * M, s);
+            if (rs != BST_OK) return rs;
+        }
     }
     if (nl > 1) {
         for (int l = 0; l < nl; ++l) {

@@ -69,7 +69,7 @@ bst_status_t bst_launch_forward_chunked(bst_plan_s* p, const float* sino, int sl
 bst_status_t bst_launch_forward(bst_plan_s* p, const float* sino, int slices, int mode, const float* g, float* vol,
                                 void* ws, size_t ws_bytes, cudaStream_t st) {
     const int pairs = (slices + 1) / 2;
-    const int chunk = std::min(pairs, p->chunk_pairs);
+    const int chunk = bsth::fwd_chunk(p, pairs, p->chunk_pairs);
     const int lanes = (int)std::min<size_t>(bsth::kMaxLanes, ws_bytes / ((size_t)chunk * bsth::fwd_bytes_per_pair(p)));
     return bst_launch_forward_chunked(p, sino, slices, mode, g, vol, ws, st, p->chunk_pairs, lanes);
 }
@@ -97,7 +97,7 @@ extern "C" bst_status_t bst_fbp_prep(bst_plan_t p, const float* d_sino, int slic
     const uintptr_t a0 = (uintptr_t)d_sino, b0 = (uintptr_t)d_volume;
     if (a0 < b0 + nv && b0 < a0 + ns) return BST_ERR_INVALID_ARGUMENT;
     if (!d_ws || ws_bytes < bst_workspace_bytes(p, slices)) return BST_ERR_WORKSPACE_TOO_SMALL;
-    const int chunk = std::min((slices + 1) / 2, p->chunk_pairs);
+    const int chunk = bsth::fwd_chunk(p, (slices + 1) / 2, p->chunk_pairs);
     const size_t lane = (size_t)chunk * bsth::fwd_bytes_per_pair(p);
     const int lanes = (int)std::min<size_t>(bsth::kMaxLanes, (ws_bytes - bsth::prep_table_bytes(p)) / lane);
     float2* cw = (float2*)((char*)d_ws + lanes * lane);

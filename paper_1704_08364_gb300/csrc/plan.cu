@@ -217,9 +217,19 @@ bst_status_t bst_plan_create(bst_plan_t* out, int rays, int angles, const float*
             return gs;
         }
     }
-    const size_t per_pair = bsth::fwd_bytes_per_pair(p);
+    // The launch shape a plan starts with: interleaved groups, chunks of 64 MiB
+    // of workspace but at least 8 pairs (whole groups), which fill several waves
+    // of blocks at every length; pair-fastest gridding where a geometry table (6
+    // M^2 bytes) is too large to stay in L2 beside Z.  Against the packed layout
+    // with chunks of 64 MiB: 15 x 1201 x 1536 backprojection 1220 -> 815 us.
+    // Chunks of 2, 4, 8, 16 pairs: 64 x 2048 x 2048 4421, 4354, 4299, 4258 us; 512 x
+    // 512 x 512 2360, 1751, 1656, 1651 us.
     const size_t budget = (size_t)64 << 20;
-    p->chunk_pairs = (int)std::max<size_t>(1, std::min<size_t>(256, budget / per_pair));
+    const size_t fit = std::min<size_t>(256, budget / bsth::fwd_bytes_per_pair(p));
+    p->chunk_pairs = (int)std::max<size_t>(8, fit & ~(size_t)7);
+    p->fwd_layout = BST_LAYOUT_INTERLEAVED;
+    p->grid_xchg = 1;
+    p->pair_fast = M >= 2048;
     p->chunk_default = p->chunk_pairs;
     // bst_fbp_noalloc's set-up for this device (a failure here leaves the
     // plan usable; bst_fbp_noalloc then retries and reports it)
@@ -240,7 +250,7 @@ int bst_plan_fft_length(bst_plan_t p) { return p ? p->M : 0; }
 size_t bst_workspace_bytes(bst_plan_t p, int slices) {
     if (!p || slices <= 0) return 0;
     const int pairs = (slices + 1) / 2;
-    const int chunk = std::min(pairs, p->chunk_pairs);
+    const int chunk = bsth::fwd_chunk(p, pairs, p->chunk_pairs);
     const int nchunks = (pairs + chunk - 1) / chunk;
     const int lanes = std::min(std::min(nchunks, bsth::kMaxLanes), std::max(p->max_lanes, 1));   // chunks in flight
     return (size_t)lanes * chunk * bsth::fwd_bytes_per_pair(p) + bsth::prep_table_bytes(p);
@@ -340,7 +350,8 @@ int bst_plan_get_schedule(bst_plan_t p) { return p ? p->maxr : 0; }
 bst_status_t bst_plan_set_forward_config(bst_plan_t p, const bst_fwd_config_t* c) {
     if (!p || !c) return BST_ERR_INVALID_ARGUMENT;
     if ((c->max_radix != 8 && c->max_radix != 16) ||
-        (c->layout != BST_LAYOUT_PACKED && c->layout != BST_LAYOUT_PAIRED) || c->chunk_pairs < 1 ||
+        (c->layout != BST_LAYOUT_PACKED && c->layout != BST_LAYOUT_PAIRED && c->layout != BST_LAYOUT_INTERLEAVED) ||
+        c->chunk_pairs < 1 ||
         c->chunk_pairs > 256 || (c->pair_fast != 0 && c->pair_fast != 1) || c->max_lanes < 1 ||
         c->max_lanes > bsth::kMaxLanes || (c->grid_xchg != 0 && c->grid_xchg != 1))
         return BST_ERR_INVALID_ARGUMENT;
@@ -364,35 +375,25 @@ bst_status_t bst_plan_get_forward_config(bst_plan_t p, bst_fwd_config_t* c) {
     return BST_OK;
 }
 
-// The candidate launch shapes of the autotuner: radix 16 or 8, the packed or
-// (bilinear plans) paired spectrum layout, for the paired layout the gather
-// through shared memory or into registers, and the default chunk in column-fastest
-// order or pair-fastest order; where the default chunk is a single pair (the
-// workspace of one pair exceeds L2), also chunks of 2, 4 and 8 pairs: the
-// launches then fill more waves of blocks, at the price of a workspace (and
-// intermediates in HBM) that grows with the chunk.  The lane count stays the
-// plan's.
+// The candidate launch shapes of the autotuner: for bilinear plans the
+// interleaved layout (where the length has it) and the paired one; half the
+// default chunk, the default and twice it (a larger chunk fills more waves of
+// blocks, a smaller one keeps the intermediates in L2); either block order.  The
+// lane count stays the plan's.  Radix 8 (never fewer passes), the packed layout
+// and the paired gather through shared memory measured slower at every length
+// and are left to bst_plan_set_forward_config.
 static std::vector<bst_fwd_config_t> tune_candidates(const bst_plan_s* p) {
     std::vector<bst_fwd_config_t> out;
-    const int layouts = p->grid_kind == BST_GRID_BILINEAR ? 3 : 1;   // packed, paired, paired + exchange
-    for (int r : {16, 8})
-        for (int lg = 0; lg < layouts; ++lg) {
-            const int l = lg == 0 ? BST_LAYOUT_PACKED : BST_LAYOUT_PAIRED;
-            bst_fwd_config_t c{r, l, p->chunk_default, 0, p->max_lanes, lg == 2 ? 1 : 0};
-            out.push_back(c);
-            if (p->chunk_default == 1) {
-                for (int ch : {2, 4, 8}) {
-                    c.chunk_pairs = ch;
-                    c.pair_fast = 0;
-                    out.push_back(c);
-                    c.pair_fast = 1;
-                    out.push_back(c);
-                }
-            } else {
-                c.pair_fast = 1;
-                out.push_back(c);
-            }
-        }
+    std::vector<int> layouts;
+    if (p->grid_kind != BST_GRID_BILINEAR) {
+        layouts = {BST_LAYOUT_PACKED};
+    } else {
+        if (bsth::inter_pairs_of(p->M) > 1) layouts.push_back(BST_LAYOUT_INTERLEAVED);
+        layouts.push_back(BST_LAYOUT_PAIRED);
+    }
+    for (int l : layouts)
+        for (int ch : {p->chunk_default / 2, p->chunk_default, std::min(256, 2 * p->chunk_default)})
+            for (int pf : {0, 1}) out.push_back(bst_fwd_config_t{16, l, ch, pf, p->max_lanes, 1});
     return out;
 }
 
@@ -403,8 +404,8 @@ bst_status_t bst_plan_autotune(bst_plan_t p, int slices, int* chosen) {
         const size_t per = (size_t)p->V * p->N * sizeof(float);
         slices = (int)std::max<size_t>(4, std::min<size_t>(4096, (((size_t)256 << 20) / per) & ~(size_t)1));
     }
-    // at least two chunks of the largest candidate on each lane
-    slices = std::max(slices, p->chunk_default == 1 ? 2 * 2 * 8 * 2 : 4);
+    // at least one chunk of the largest candidate on each lane
+    slices = std::max(slices, 2 * 2 * std::min(256, 2 * p->chunk_default));
     bst_fwd_config_t old{};
     bst_plan_get_forward_config(p, &old);
     const std::vector<bst_fwd_config_t> cand = tune_candidates(p);
