@@ -28,9 +28,20 @@ namespace bst {
 // with a factor i takes the scalar form (cadd_si), whose operands need no
 // swapping.  At 2048 x 2048, pad 2: ray kernel 27.0 -> 25.4 us a pair, gridding
 // 90.3 -> 88.9, row kernel 24.1 -> 24.8.
+// (The scalar branch only lets host programs that check the tables include this
+// header without naming the architecture.)
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return __fmul2_rn(a, make_float2(s, s)); }
+#else
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 c) {
+    return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
+}
+__device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+#endif
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return cfma(b, make_float2(-1.f, -1.f), a); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -75,7 +86,7 @@ template <bool INV> struct Dft<3, INV> {
     __device__ __forceinline__ static void run(float2* a) {
         const float2 t = cadd(a[1], a[2]);
         const float2 u = csub(a[1], a[2]);
-        const float2 m = __ffma2_rn(make_float2(-0.5f, -0.5f), t, a[0]);
+        const float2 m = cfma(make_float2(-0.5f, -0.5f), t, a[0]);
         const float2 v = cscale(u, BST_H3);
         a[0] = cadd(a[0], t);
         a[1] = cadd_si<INV>(m, v);
