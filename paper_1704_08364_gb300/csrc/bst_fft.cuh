@@ -160,6 +160,18 @@ template <bool INV> struct Dft<16, INV> {
     }
 };
 
+// ---- kernels in a row ------------------------------------------------------
+//
+// At the start of a kernel that may be launched with programmatic stream
+// serialization: lets the next kernel of the stream be set up while this one
+// runs, then waits until the previous one is complete and its writes are
+// visible.  Every kernel of the forward path calls it first, so completion is
+// transitive.  Nothing without that launch attribute.
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---- radix schedule --------------------------------------------------------
 
 __host__ __device__ constexpr int ilog2c(int x) { return x <= 1 ? 0 : 1 + ilog2c(x / 2); }
@@ -221,6 +233,8 @@ struct WorkerSync {
     int n;    // threads of the worker
     __device__ __forceinline__ void operator()() const {
         asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+    }
+};
     }
 };
 
