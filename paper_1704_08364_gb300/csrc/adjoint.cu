@@ -250,7 +250,8 @@ struct SinoCrop {
 // the next lane by a shuffle, across warps through `edge`).  Reading every cell
 // once per sample and pair instead (four times, 8 bytes of each 32-byte sector)
 // waited on the list-to-point chains (16 stall cycles per issue): 486 us for
-// the 8 pairs of 16 x 1024 x 1024, 280 us with this form.  What bounds it
+// the 8 pairs of 16 x 1024 x 1024, 280 us with this form and 212 us with the next
+// cell's list bounds read ahead.  What bounds it
 // now is the latency and sector traffic of the point reads from L2.
 template <int M, int TPL, int LINES, int P>
 __global__ void __launch_bounds__(TPL * LINES, 1024 / (TPL * LINES))
@@ -266,6 +267,18 @@ __global__ void __launch_bounds__(TPL * LINES, 1024 / (TPL * LINES))
     const int j0 = blockIdx.x * L;
     const float2* Xp = X + (size_t)blockIdx.y * P * M * M;
     const float2 zero = make_float2(0.f, 0.f);
+    // the list bounds of the next cell are read while this one is worked on
+    auto bounds = [&](int k, int b, int& lo, int& hi) {
+        const int J = j0 - 1 + b;
+        lo = hi = 0;
+        if (k < M && J < V) {
+            const int cell = (J + 1) * M + k;
+            lo = __ldg(cl.start + cell);
+            hi = __ldg(cl.start + cell + 1);
+        }
+    };
+    int sn, en;
+    bounds(tid, 0, sn, en);
 #pragma unroll 1
     for (int k0 = 0; k0 < M; k0 += NT) {
         const int kappa = k0 + tid;
@@ -280,10 +293,11 @@ __global__ void __launch_bounds__(TPL * LINES, 1024 / (TPL * LINES))
             float2 own1[P], hi1[P];
 #pragma unroll
             for (int p = 0; p < P; ++p) own1[p] = hi1[p] = zero;
-            if (act && J < V) {
-                const int cell = (J + 1) * M + kappa;
-                const int e = __ldg(cl.start + cell + 1);
-                for (int i = __ldg(cl.start + cell); i < e; ++i) {
+            {
+                const int e = en;
+                int i = sn;
+                bounds(b == L ? kappa + NT : kappa, b == L ? 0 : b + 1, sn, en);
+                for (; i < e; ++i) {
                     const float2 fw = __ldg(cl.w + i);
                     float2 x[P];
                     load_point<P>(Xp, __ldg(cl.pts + i), x);
