@@ -88,18 +88,19 @@ __global__ void __launch_bounds__(4 * TPL * TPC)
     extern __shared__ float2 smem[];
     const int pl = blockIdx.y;
     const int tile = threadIdx.x / (4 * TPL);
-    const int w = threadIdx.x % (4 * TPL);
-    const int line = w & 3, t = w >> 2;
+    // the image rows are read one by one, T is written with the four rows interleaved
+    const LineMap m = ray_lines<M, TPL, 4, 16, true>(threadIdx.x % (4 * TPL));
     const int rb = blockIdx.x * TPC + tile;
-    const int r = rb * 4 + line;
+    const int r = rb * 4 + m.line0;
     const bool live = r < N;
     const int rr = live ? r : 0;
     const int sa = 2 * (pair0 + pl), sb = sa + 1;
-    ImgRowSrc src{vol + ((size_t)sa * N + rr) * N, sb < slices ? vol + ((size_t)sb * N + rr) * N : nullptr, N, M,
-                  live};
-    TileDst dst{T + (size_t)pl * ((N + 3) / 4) * 4 * M, M, rb, line, rb * 4 < N};
-    SmemLine sm{smem + (tile * 4 + line) * adj_row_stride<M>()};
-    fft_line<M, TPL, false>(t, src, dst, sm, tw);
+    const ImgRowSrc src{vol + ((size_t)sa * N + rr) * N, sb < slices ? vol + ((size_t)sb * N + rr) * N : nullptr, N, M,
+                        live};
+    const TileDst dst{T + (size_t)pl * ((N + 3) / 4) * 4 * M, M, rb, m.line1, rb * 4 < N};
+    float2* base = smem + tile * 4 * adj_row_stride<M>();
+    fft_line_remap<M, TPL, false, 16, false, false>(m.t0, src, SmemLine{base + m.line0 * adj_row_stride<M>()}, m.t1, dst,
+                                  SmemLine{base + m.line1 * adj_row_stride<M>()}, tw);
 }
 
 // ---------------------------------------------------------------------------

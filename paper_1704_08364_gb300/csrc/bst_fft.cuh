@@ -457,11 +457,12 @@ __device__ __forceinline__ void stockham_pass(int t, const Src& src, const Dst& 
 }
 
 // Run passes PIDX.. of the length-M transform.  Pass 0 reads `src`, the last
-// pass writes `dst`; the others go through the shared-memory line `sm`.
+// pass writes `dst`; the others go through the shared-memory line `sm`.  The last
+// pass runs as thread tl of the line sml (t, sm unless the maps change there).
 // Every thread that `sync` covers must call this (it contains barriers).
 template <int M, int TPL, bool INV, int MAXR, int PIDX, int NS, bool TWT, class Src, class Dst, class SYNC>
-__device__ __forceinline__ void fft_run(int t, const Src& src, const Dst& dst, const SmemLine& sm,
-                                        const float2* __restrict__ tw, const SYNC& sync) {
+__device__ __forceinline__ void fft_run(int t, const Src& src, const Dst& dst, const SmemLine& sm, int tl,
+                                        const SmemLine& sml, const float2* __restrict__ tw, const SYNC& sync) {
     constexpr int R = radix_of(M, PIDX, MAXR);
     constexpr bool LAST = (NS * R == M);
     constexpr int TB = pass_tab_base(M, MAXR, PIDX);
@@ -471,15 +472,15 @@ __device__ __forceinline__ void fft_run(int t, const Src& src, const Dst& dst, c
         } else {
             stockham_pass<M, R, NS, TPL, INV, TWT, TB>(t, src, sm, tw, Src::kSmem, sync);
             sync();
-            fft_run<M, TPL, INV, MAXR, PIDX + 1, NS * R, TWT>(t, src, dst, sm, tw, sync);
+            fft_run<M, TPL, INV, MAXR, PIDX + 1, NS * R, TWT>(t, src, dst, sm, tl, sml, tw, sync);
         }
     } else {
         if constexpr (LAST) {
-            stockham_pass<M, R, NS, TPL, INV, TWT, TB>(t, sm, dst, tw, Dst::kSmem, sync);
+            stockham_pass<M, R, NS, TPL, INV, TWT, TB>(tl, sml, dst, tw, Dst::kSmem, sync);
         } else {
             stockham_pass<M, R, NS, TPL, INV, TWT, TB>(t, sm, sm, tw, true, sync);
             sync();
-            fft_run<M, TPL, INV, MAXR, PIDX + 1, NS * R, TWT>(t, src, dst, sm, tw, sync);
+            fft_run<M, TPL, INV, MAXR, PIDX + 1, NS * R, TWT>(t, src, dst, sm, tl, sml, tw, sync);
         }
     }
 }
@@ -489,7 +490,32 @@ __device__ __forceinline__ void fft_run(int t, const Src& src, const Dst& dst, c
 template <int M, int TPL, bool INV, int MAXR = 16, bool TWT = false, class Src, class Dst, class SYNC = BlockSync>
 __device__ __forceinline__ void fft_line(int t, const Src& src, const Dst& dst, const SmemLine& sm,
                                          const float2* __restrict__ tw, const SYNC& sync = SYNC()) {
-    fft_run<M, TPL, INV, MAXR, 0, 1, TWT>(t, src, dst, sm, tw, sync);
+    fft_run<M, TPL, INV, MAXR, 0, 1, TWT>(t, src, dst, sm, t, sm, tw, sync);
+}
+
+// Two thread-to-line maps for one transform: the first pass (LATE: all but the
+// last) runs as thread t0 of a line whose source is src and whose storage is sm0,
+// the others as thread t1 of a line with storage sm1 and sink dst.  A block may
+// so read its lines one way (whole segments of a row, say) and write them another
+// way (several lines interleaved), each coalesced.  With interleaved lines the
+// base-table twiddles of a warp are those of fewer butterflies, so a transform
+// without per-pass tables stays interleaved as long as it can.  `sync` covers the
+// threads of all the lines.  A transform of a single pass cannot change maps
+// (fft_remaps: then t0 = t1, sm0 = sm1).
+template <int M, int MAXR = 16> __host__ __device__ constexpr bool fft_remaps() { return radix_of(M, 0, MAXR) < M; }
+template <int M, int TPL, bool INV, int MAXR, bool TWT, bool LATE, class Src, class Dst, class SYNC = BlockSync>
+__device__ __forceinline__ void fft_line_remap(int t0, const Src& src, const SmemLine& sm0, int t1, const Dst& dst,
+                                               const SmemLine& sm1, const float2* __restrict__ tw,
+                                               const SYNC& sync = SYNC()) {
+    constexpr int R = radix_of(M, 0, MAXR);
+    static_assert(!Src::kSmem, "a source outside the lines");
+    if constexpr (LATE || !fft_remaps<M, MAXR>()) {
+        fft_run<M, TPL, INV, MAXR, 0, 1, TWT>(t0, src, dst, sm0, t1, sm1, tw, sync);
+    } else {
+        stockham_pass<M, R, 1, TPL, INV, TWT, 0>(t0, src, sm0, tw, false, sync);
+        sync();
+        fft_run<M, TPL, INV, MAXR, 1, R, TWT>(t1, src, dst, sm1, t1, sm1, tw, sync);
+    }
 }
 
 // The transform of a line whose values thread t already holds in registers,
@@ -499,9 +525,11 @@ __device__ __forceinline__ void fft_line(int t, const Src& src, const Dst& dst, 
 // directly and only its outputs go to the shared-memory line `sm`; the later
 // passes are those of fft_line.  Call with every thread of the block; `sm`
 // must be free for writing (the caller's barrier).
+// sm1, t1: storage and thread of the later passes, as in fft_line_remap.
 template <int M, int TPL, bool INV, int MAXR = 16, class Dst, class SYNC = BlockSync, bool TWT = false>
-__device__ __forceinline__ void fft_line_regs(int t, float2 (&x)[M / TPL], const Dst& dst, const SmemLine& sm,
-                                              const float2* __restrict__ tw, const SYNC& sync = SYNC()) {
+__device__ __forceinline__ void fft_line_regs(int t, float2 (&x)[M / TPL], const Dst& dst, const SmemLine& sm, int t1,
+                                              const SmemLine& sm1, const float2* __restrict__ tw,
+                                              const SYNC& sync = SYNC()) {
     constexpr int R = radix_of(M, 0, MAXR);
     constexpr int NB = M / R;
     static_assert(NB % TPL == 0, "one or more whole first-pass butterflies per thread");
@@ -533,8 +561,13 @@ __device__ __forceinline__ void fft_line_regs(int t, float2 (&x)[M / TPL], const
     }
     if constexpr (R < M) {
         sync();
-        fft_run<M, TPL, INV, MAXR, 1, R, TWT>(t, sm, dst, sm, tw, sync);
+        fft_run<M, TPL, INV, MAXR, 1, R, TWT>(t1, sm1, dst, sm1, t1, sm1, tw, sync);
     }
+}
+template <int M, int TPL, bool INV, int MAXR = 16, class Dst, class SYNC = BlockSync, bool TWT = false>
+__device__ __forceinline__ void fft_line_regs(int t, float2 (&x)[M / TPL], const Dst& dst, const SmemLine& sm,
+                                              const float2* __restrict__ tw, const SYNC& sync = SYNC()) {
+    fft_line_regs<M, TPL, INV, MAXR, Dst, SYNC, TWT>(t, x, dst, sm, t, sm, tw, sync);
 }
 
 // signed frequency of natural-order index p

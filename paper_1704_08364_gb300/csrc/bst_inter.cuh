@@ -88,17 +88,21 @@ __global__ void __launch_bounds__(inter_ray_threads<M>(), 1024 / inter_ray_threa
     constexpr int TPL = tpl_of<M>(), P = inter_pairs<M>(), LP = inter_lanes<P>();
     extern __shared__ float2 smem[];
     chain_begin();
-    const int l = threadIdx.x % LP, t = (threadIdx.x / LP) % TPL, row = threadIdx.x / (LP * TPL);
-    const int grp = blockIdx.y / (P / LP), p = (blockIdx.y % (P / LP)) * LP + l;
+    // the rays are read pair by pair, the spectrum is written with the pairs interleaved
+    const int row = threadIdx.x / (LP * TPL);
+    const LineMap m = ray_lines<M, TPL, LP, MAXR, true>(threadIdx.x % (LP * TPL));
+    const int grp = blockIdx.y / (P / LP), pb = (blockIdx.y % (P / LP)) * LP;
     const int j = blockIdx.x * inter_ray_rows<M>() + row;
     const bool live = j < V;
     const int jj = live ? j : 0;
-    const int sa = 2 * (pair0 + grp * P + p), sb = sa + 1;
+    const int sa = 2 * (pair0 + grp * P + pb + m.line0), sb = sa + 1;
     const bool hb = sb < slices;
     const float* ya = sino + ((size_t)sa * V + jj) * N;
     const float* yb = hb ? sino + ((size_t)sb * V + jj) * N : nullptr;
     float2* z = Z + (size_t)grp * V * M * P;
-    const SmemLine sm{smem + (row * LP + l) * inter_stride<M>(LP)};
+    const int p = pb + m.line1;
+    const SmemLine sm0{smem + (row * LP + m.line0) * inter_stride<M>(LP)};
+    const SmemLine sm1{smem + (row * LP + m.line1) * inter_stride<M>(LP)};
     if constexpr (PREP) {
         const PrepRays rays{ya,
                             yb,
@@ -109,12 +113,12 @@ __global__ void __launch_bounds__(inter_ray_threads<M>(), 1024 / inter_ray_threa
                             pa.win};
         const InterDstPrep<M, P> dst{z, jj, p, pa.cw, live};
         float2 x[M / TPL];
-        prep_gather<M, TPL, NC>(rays, t, N, live, x);
-        fft_line_regs<M, TPL, false, MAXR, InterDstPrep<M, P>, BlockSync, true>(t, x, dst, sm, tw);
+        prep_gather<M, TPL, NC>(rays, m.t0, N, live, x);
+        fft_line_regs<M, TPL, false, MAXR, InterDstPrep<M, P>, BlockSync, true>(m.t0, x, dst, sm0, m.t1, sm1, tw);
     } else {
         const RaySrc<NC> src{ya, yb, N, M, live};
         const InterDst<M, P> dst{z, jj, p, g, mode, two_alpha, live};
-        fft_line<M, TPL, false, MAXR, true>(t, src, dst, sm, tw);
+        fft_line_remap<M, TPL, false, MAXR, true, false>(m.t0, src, sm0, m.t1, dst, sm1, tw);
     }
 }
 
@@ -286,17 +290,21 @@ __global__ void __launch_bounds__(4 * tpl_of<M>() * inter_row_tiles<M>(), 1024 /
     constexpr int TPL = tpl_of<M>(), P = inter_pairs<M>(), LP = inter_lanes<P>(), G = inter_rows<P>();
     extern __shared__ float2 smem[];
     chain_begin();
-    const int tile = threadIdx.x / (4 * TPL), l = threadIdx.x % 4, t = (threadIdx.x / 4) % TPL;
-    const int grp = blockIdx.y / (P / LP), p = (blockIdx.y % (P / LP)) * LP + l % LP;
-    const int r = (blockIdx.x * inter_row_tiles<M>() + tile) * (4 / LP) + l / LP;
-    const bool live = r < N;
-    const int rr = live ? r : 0;
-    const int sa = 2 * (pair0 + grp * P + p), sb = sa + 1;
-    const InterTileSrc<M, P> src{T + (size_t)grp * N * M * P + (size_t)(rr / G) * M * G * P + (rr % G) * P + p};
-    const VolDst<NC> dst{vol + ((size_t)sa * N + rr) * N, sb < slices ? vol + ((size_t)sb * N + rr) * N : nullptr,
-                         N, M, scale, live, nullptr};
-    const SmemLine sm{smem + (tile * 4 + l) * row_line_stride<M>()};
-    fft_line<M, TPL, true, MAXR>(t, src, dst, sm, tw);
+    const int tile = threadIdx.x / (4 * TPL);
+    const LineMap m = tile_lines<M, TPL, 4, MAXR>(threadIdx.x % (4 * TPL));
+    const int grp = blockIdx.y / (P / LP), pb = (blockIdx.y % (P / LP)) * LP;
+    const int rb = (blockIdx.x * inter_row_tiles<M>() + tile) * (4 / LP);
+    // line l: pair pb + l % LP of row rb + l / LP
+    const int ra = rb + m.line0 / LP, pa = pb + m.line0 % LP;
+    const int r = rb + m.line1 / LP, sa = 2 * (pair0 + grp * P + pb + m.line1 % LP), sb = sa + 1;
+    const int rr = ra < N ? ra : 0;
+    const InterTileSrc<M, P> src{T + (size_t)grp * N * M * P + (size_t)(rr / G) * M * G * P + (rr % G) * P + pa};
+    const size_t at = (size_t)(r < N ? r : 0) * N;
+    const VolDst<NC> dst{vol + (size_t)sa * N * N + at, sb < slices ? vol + (size_t)sb * N * N + at : nullptr,
+                         N, M, scale, r < N, nullptr};
+    float2* base = smem + tile * 4 * row_line_stride<M>();
+    fft_line_remap<M, TPL, true, MAXR, false, true>(m.t0, src, SmemLine{base + m.line0 * row_line_stride<M>()}, m.t1, dst,
+                                       SmemLine{base + m.line1 * row_line_stride<M>()}, tw);
 }
 
 }  // namespace bst

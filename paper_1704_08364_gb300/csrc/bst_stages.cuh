@@ -365,6 +365,33 @@ struct SpecDstPrep {
 // lanes of two lines at the same offset do not share a bank.
 template <int M, bool ILV> __host__ __device__ constexpr int ray_line_stride() { return smem_line_len(M) + (ILV ? 8 : 0); }
 
+// Thread-to-line maps of a unit (fft_line_remap): line0, t0 of the first pass,
+// line1, t1 of the others.
+struct LineMap {
+    int line0, t0, line1, t1;
+};
+// of LPC ray lines: the rays are read line by line, the spectrum is written with
+// the lines interleaved over the lanes (ILV)
+template <int M, int TPL, int LPC, int MAXR, bool ILV>
+__device__ __forceinline__ LineMap ray_lines(int tid) {
+    LineMap m{tid / TPL, tid % TPL, ILV ? tid % LPC : tid / TPL, ILV ? tid / LPC : tid % TPL};
+    if (!fft_remaps<M, MAXR>()) {
+        m.line0 = m.line1;
+        m.t0 = m.t1;
+    }
+    return m;
+}
+// of a tile of L lines: read interleaved (the lines of a piece of T), written line by line
+template <int M, int TPL, int L, int MAXR>
+__device__ __forceinline__ LineMap tile_lines(int w) {
+    LineMap m{w % L, w / L, w / TPL, w % TPL};
+    if (!fft_remaps<M, MAXR>()) {
+        m.line1 = m.line0;
+        m.t1 = m.t0;
+    }
+    return m;
+}
+
 // ray_unit with the pre-reconstruction stages (slice rows da/db, fa/fb of the
 // dark and flat fields, or null)
 template <int M, int TPL, int LPC, int MAXR, int NC = 0, bool ILV = false>
@@ -372,16 +399,16 @@ __device__ __forceinline__ void ray_unit_prep(float2* smem, int j0, int V, int N
                                               const float* __restrict__ yb, const float* da, const float* db,
                                               const float* fa, const float* fb, const PrepArgs& pa, int mode,
                                               float2* __restrict__ Zp, const float2* __restrict__ tw) {
-    const int line = ILV ? threadIdx.x % LPC : threadIdx.x / TPL, t = ILV ? threadIdx.x / LPC : threadIdx.x % TPL;
-    const int j = j0 + line;
-    const bool live = j < V;
-    const int jj = live ? j : 0;
-    const PrepRays rays{ya + (size_t)jj * N, yb ? yb + (size_t)jj * N : nullptr, da, db, fa, fb, pa.win};
-    const SpecDstPrep dst{Zp, jj, V, pa.cw, M, mode, live};
-    const SmemLine sm{smem + line * ray_line_stride<M, ILV>()};
+    const LineMap m = ray_lines<M, TPL, LPC, MAXR, ILV>(threadIdx.x);
+    const int ja = j0 + m.line0, jb = j0 + m.line1;   // of the rays, of the spectrum
+    const size_t at = (size_t)(ja < V ? ja : 0) * N;
+    const PrepRays rays{ya + at, yb ? yb + at : nullptr, da, db, fa, fb, pa.win};
+    const SpecDstPrep dst{Zp, jb < V ? jb : 0, V, pa.cw, M, mode, jb < V};
+    constexpr int LS = ray_line_stride<M, ILV>();
     float2 x[M / TPL];
-    prep_gather<M, TPL, NC>(rays, t, N, live, x);
-    fft_line_regs<M, TPL, false, MAXR, SpecDstPrep, BlockSync, true>(t, x, dst, sm, tw);
+    prep_gather<M, TPL, NC>(rays, m.t0, N, ja < V, x);
+    fft_line_regs<M, TPL, false, MAXR, SpecDstPrep, BlockSync, true>(m.t0, x, dst, SmemLine{smem + m.line0 * LS}, m.t1,
+                                                                     SmemLine{smem + m.line1 * LS}, tw);
 }
 
 // P2 + P3 + P4 for lines j0 .. j0 + LPC - 1 of one slice pair (TPL * LPC
@@ -395,14 +422,14 @@ __device__ __forceinline__ void ray_unit(float2* smem, int j0, int V, int N, con
                                          float two_alpha, float2* __restrict__ Zp, const float2* __restrict__ tw,
                                          const SYNC& sync = SYNC(), int tid = -1) {
     if (tid < 0) tid = threadIdx.x;
-    const int line = ILV ? tid % LPC : tid / TPL, t = ILV ? tid / LPC : tid % TPL;
-    const int j = j0 + line;
-    const bool live = j < V;
-    const int jj = live ? j : 0;
-    RaySrc<NC> src{ya + (size_t)jj * N, yb ? yb + (size_t)jj * N : nullptr, N, M, live};
-    SpecDst dst{Zp, jj, V, g, M, mode, two_alpha, live};
-    SmemLine sm{smem + line * ray_line_stride<M, ILV>()};
-    fft_line<M, TPL, false, MAXR, TWT>(t, src, dst, sm, tw, sync);
+    const LineMap m = ray_lines<M, TPL, LPC, MAXR, ILV>(tid);
+    const int ja = j0 + m.line0, jb = j0 + m.line1;   // of the rays, of the spectrum
+    const size_t at = (size_t)(ja < V ? ja : 0) * N;
+    const RaySrc<NC> src{ya + at, yb ? yb + at : nullptr, N, M, ja < V};
+    const SpecDst dst{Zp, jb < V ? jb : 0, V, g, M, mode, two_alpha, jb < V};
+    constexpr int LS = ray_line_stride<M, ILV>();
+    fft_line_remap<M, TPL, false, MAXR, TWT, false>(m.t0, src, SmemLine{smem + m.line0 * LS}, m.t1, dst,
+                                             SmemLine{smem + m.line1 * LS}, tw, sync);
 }
 
 // P0 + P5 + column P6 for column pairs q0 .. q0 + CPC - 1 (blockDim = TPL * CPC):
@@ -789,16 +816,15 @@ __device__ __forceinline__ void row_unit(float2* smem, int rb0, int N, const flo
     static_assert(RPT == 4 || RPT == 2, "rows per tile");
     if (tid < 0) tid = threadIdx.x;
     const int tile = tid / (RPT * TPL);
-    const int w = tid % (RPT * TPL);
-    const int line = w % RPT, t = w / RPT;
-    const int r = (rb0 + tile) * RPT + line;
-    const bool live = r < N;
-    const int rr = live ? r : 0;
-    TileSrc src{Tp, M, rr, live};
-    VolDst<NC> dst{va + (size_t)rr * N, vb ? vb + (size_t)rr * N : nullptr, N, M,
-               dk ? scale * __ldg(dk + rr) : scale, live, dk};
-    SmemLine sm{smem + (tile * RPT + line) * row_line_stride<M>()};
-    fft_line<M, TPL, true, MAXR, TWT>(t, src, dst, sm, tw, sync);
+    const LineMap m = tile_lines<M, TPL, RPT, MAXR>(tid % (RPT * TPL));
+    const int r0 = (rb0 + tile) * RPT + m.line0, r1 = (rb0 + tile) * RPT + m.line1;
+    const TileSrc src{Tp, M, r0 < N ? r0 : 0, r0 < N};
+    const int rr = r1 < N ? r1 : 0;
+    const VolDst<NC> dst{va + (size_t)rr * N, vb ? vb + (size_t)rr * N : nullptr, N, M,
+                         dk ? scale * __ldg(dk + rr) : scale, r1 < N, dk};
+    float2* base = smem + tile * RPT * row_line_stride<M>();
+    fft_line_remap<M, TPL, true, MAXR, TWT, true>(m.t0, src, SmemLine{base + m.line0 * row_line_stride<M>()}, m.t1, dst,
+                                            SmemLine{base + m.line1 * row_line_stride<M>()}, tw, sync);
 }
 
 }  // namespace bst
