@@ -4,7 +4,8 @@
 //   Z per group of P pairs: [V][M/2][2][P] complex64, slot k of a row holding
 //     Z[+k] of the P pairs and then Z[-k] of the P pairs (bin 0 fills both; the
 //     Nyquist bin, weight 0, is not stored): one bilinear tap of all P pairs and
-//     of a point and its mirror is one contiguous piece of 16 P bytes.
+//     of a point and its mirror is one contiguous piece of 16 P bytes (for P = 2
+//     two halves of a 64-byte piece, inter_slot).
 //   T per group: [N/G][M][G][P] complex64, G = 8 / P rows: a column writes
 //     64-byte pieces, a row tile reads 32-byte sectors.  (32-byte pieces for P = 2
 //     read faster and write slower: 64 x 2048 x 2048 4257 -> 4341 us.)
@@ -35,16 +36,23 @@ template <int P> __host__ __device__ constexpr int inter_lanes() { return P < 4 
 // stride between lines whose lanes alternate over n lines: skewed by 32 / n banks
 template <int M> __host__ __device__ constexpr int inter_stride(int n) { return smem_line_len(M) + 16 / n; }
 
+// Place of slot k, sign s (0: +k, 1: -k) in a row, in complex values: [k][s][P],
+// for P = 2 [k / 2][s][k % 2][P], so that the ray kernel writes whole sectors there
+// too (consecutive bins of one sign).
+template <int P> __device__ __forceinline__ int inter_slot(int k, int s) {
+    return P == 2 ? (k >> 1) * 8 + s * 4 + (k & 1) * 2 : (k * 2 + s) * P;
+}
+
 // store of the weighted spectrum value of bin k into slot |k| of row j
 template <int M, int P>
 __device__ __forceinline__ void inter_store(float2* z, int j, int p, int k, float2 v) {
     constexpr int H = M / 2;
     float2* row = z + (size_t)j * M * P + p;
     if (k < H) {
-        row[k * 2 * P] = v;
-        if (k == 0) row[P] = v;
+        row[inter_slot<P>(k, 0)] = v;
+        if (k == 0) row[inter_slot<P>(0, 1)] = v;
     } else if (k > H) {
-        row[((M - k) * 2 + 1) * P] = v;
+        row[inter_slot<P>(M - k, 1)] = v;
     }
 }
 template <int M, int P> struct InterDst {
@@ -208,12 +216,13 @@ __global__ void __launch_bounds__(2 * inter_pairs<M>() * tpl_of<M>(), 1024 / (2 
             const int rowB = sB ? 0 : J + 1;
             const int hA = (up != sA ? 0 : 1) ^ h, hB = (up != sB ? 0 : 1) ^ h;
             const bool k1ok = ok && k0 + 1 < H;
-            const float4* pa = Zg + ((rowA * H + k0) * 2 + hA) * (P / 2);
-            const float4* pb = Zg + ((rowB * H + k0) * 2 + hB) * (P / 2);
+            const float4* pa = Zg + rowA * H * P + inter_slot<P>(k0, hA) / 2;
+            const float4* pb = Zg + rowB * H * P + inter_slot<P>(k0, hB) / 2;
+            const int up1 = P == 2 ? ((k0 & 1) ? 3 : 1) : P;   // to the next bin
             z[s][0] = ok ? __ldg(pa) : zero4;
-            z[s][1] = k1ok ? __ldg(pa + P) : zero4;
+            z[s][1] = k1ok ? __ldg(pa + up1) : zero4;
             z[s][2] = ok ? __ldg(pb) : zero4;
-            z[s][3] = k1ok ? __ldg(pb + P) : zero4;
+            z[s][3] = k1ok ? __ldg(pb + up1) : zero4;
         }
 #pragma unroll
         for (int s = 0; s < PS; ++s) {
