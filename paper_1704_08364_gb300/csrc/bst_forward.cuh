@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(TPL * LPC, (TPL * LPC <= 1024) ? 1024 / (TPL *
     k_ray_fft(const float* __restrict__ sino, int slices, int pair0, int N, int V, int mode,
               const float* __restrict__ g, float two_alpha, float2* __restrict__ Z, const float2* __restrict__ tw) {
     extern __shared__ float2 smem[];
-    chain_begin();
+    chain_begin<M>();
     const int pl = blockIdx.y;
     const int sa = 2 * (pair0 + pl), sb = sa + 1;
     ray_unit<M, TPL, LPC, MAXR, NC, BlockSync, ILV, true>(smem, blockIdx.x * LPC, V, N, sino + (size_t)sa * V * N,
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(TPL * LPC, (TPL * LPC <= 1024) ? 1024 / (TPL *
     k_ray_fft_prep(const float* __restrict__ sino, int slices, int pair0, int N, int V, PrepArgs pa, int mode,
                    float2* __restrict__ Z, const float2* __restrict__ tw) {
     extern __shared__ float2 smem[];
-    chain_begin();
+    chain_begin<M>();
     const int pl = blockIdx.y;
     const int sa = 2 * (pair0 + pl), sb = sa + 1;
     const bool hb = sb < slices;
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(TPL * CPC, (TPL * CPC <= 256) ? 1024 / (TPL * 
     k_grid_col(const float2* __restrict__ Z, int V, int N, const int* __restrict__ gJ,
                const float2* __restrict__ gF, float2* __restrict__ T, const float2* __restrict__ tw, int pair_fast) {
     extern __shared__ float2 smem[];
-    chain_begin();
+    chain_begin<M>();
     const int pl = pair_fast ? blockIdx.x : blockIdx.y;
     const int cg = pair_fast ? blockIdx.y : blockIdx.x;
     grid_unit<M, TPL, CPC, MAXR, NC>(smem, cg * CPC, V, N, Z + (size_t)pl * V * M, gJ, gF,
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(2 * TPL * CPC, (2 * TPL * CPC <= 1024) ? 1024 
                       const float2* __restrict__ gF, float2* __restrict__ T, const float2* __restrict__ tw,
                       int pair_fast) {
     extern __shared__ float2 smem[];
-    chain_begin();
+    chain_begin<M>();
     const int pl = pair_fast ? blockIdx.x : blockIdx.y;
     const int cg = pair_fast ? blockIdx.y : blockIdx.x;
     grid_unit_paired<M, TPL, CPC, MAXR, NC>(smem, cg * CPC, V, N,
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(2 * TPL, (2 * TPL <= 1024) ? 1024 / (2 * TPL) 
                     const float2* __restrict__ gF, float2* __restrict__ T, const float2* __restrict__ tw,
                     int pair_fast) {
     extern __shared__ float2 smem[];
-    chain_begin();
+    chain_begin<M>();
     const int pl = pair_fast ? blockIdx.x : blockIdx.y;
     const int cq = pair_fast ? blockIdx.y : blockIdx.x;
     grid_unit_xchg<M, TPL, MAXR, NC, PS>(smem, cq, V, N, reinterpret_cast<const float4*>(Z + (size_t)pl * V * M), gJ,
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(4 * TPL * TPC)
     k_row_ifft(const float2* __restrict__ T, int slices, int pair0, int N, float scale, float* __restrict__ vol,
                const float2* __restrict__ tw, const float* __restrict__ dk) {
     extern __shared__ float2 smem[];
-    chain_begin();
+    chain_begin<M>();
     const int pl = blockIdx.y;
     const int sa = 2 * (pair0 + pl), sb = sa + 1;
     row_unit<M, TPL, TPC, MAXR, NC>(smem, blockIdx.x * TPC, N, T + (size_t)pl * ((N + 3) / 4) * 4 * M,

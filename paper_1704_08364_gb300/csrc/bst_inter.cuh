@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(inter_ray_threads<M>(), 1024 / inter_ray_threa
                 const float* __restrict__ g, float two_alpha, float2* __restrict__ Z, const float2* __restrict__ tw) {
     constexpr int TPL = tpl_of<M>(), P = inter_pairs<M>(), LP = inter_lanes<P>();
     extern __shared__ float2 smem[];
-    chain_begin();
+    chain_begin<M>();
     // the rays are read pair by pair, the spectrum is written with the pairs interleaved
     const int row = threadIdx.x / (LP * TPL);
     const LineMap m = ray_lines<M, TPL, LP, MAXR, true>(threadIdx.x % (LP * TPL));
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(2 * inter_pairs<M>() * tpl_of<M>(), 1024 / (2 
     constexpr int PPL = M / TPL, PPT = PPL / 2;
     static_assert(TPL % RW == 0 && PPL % 4 == 0 && PPT % PS == 0, "steps of the upper and lower half rows");
     extern __shared__ float2 smem[];
-    chain_begin();
+    chain_begin<M>();
     const int grp = pair_fast ? blockIdx.x : blockIdx.y, q = pair_fast ? blockIdx.y : blockIdx.x;
     const int lane = threadIdx.x & 31, e = lane % P, w = lane >> 4;
     const int h = e / (P / 2), u = e % (P / 2);
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(4 * tpl_of<M>() * inter_row_tiles<M>(), 1024 /
                 const float2* __restrict__ tw) {
     constexpr int TPL = tpl_of<M>(), P = inter_pairs<M>(), LP = inter_lanes<P>(), G = inter_rows<P>();
     extern __shared__ float2 smem[];
-    chain_begin();
+    chain_begin<M>();
     const int tile = threadIdx.x / (4 * TPL);
     const LineMap m = tile_lines<M, TPL, 4, MAXR>(threadIdx.x % (4 * TPL));
     const int grp = blockIdx.y / (P / LP), pb = (blockIdx.y % (P / LP)) * LP;

@@ -135,7 +135,7 @@ bst_status_t launch_forward_M(bst_plan_s* p, const float* sino, int slices, int 
     // against 19.4 us.  With two lanes the other lane's blocks fill that end, and
     // blocks that only wait would keep them out; with many small chunks on one
     // stream the dearer launches (about 1 us each) bound the call.
-    const bool chain = nchunks == 1 && !p->timing;
+    const bool chain = chainable(M) && nchunks == 1 && !p->timing;
     // the three stages of np pairs from pair p0 on stream s, groups interleaved
     auto run_inter = [&](int p0, int np, float2* Z, float2* T, cudaStream_t s) {
         if constexpr (InterCfg<M>::OK) {
