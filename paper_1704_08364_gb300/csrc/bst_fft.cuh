@@ -282,8 +282,6 @@ struct WorkerSync {
         asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
     }
 };
-    }
-};
 
 // ---- line storage ----------------------------------------------------------
 
