@@ -281,6 +281,10 @@ struct WorkerSync {
     __device__ __forceinline__ void operator()() const {
         asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
     }
+    // group g (of at most four) of worker id 1 or 2: its own barrier for threads of them
+    __device__ __forceinline__ WorkerSync group(int g, int threads) const {
+        return WorkerSync{3 + 4 * (id - 1) + g, threads};
+    }
 };
 
 // ---- line storage ----------------------------------------------------------

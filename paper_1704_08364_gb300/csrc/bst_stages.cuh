@@ -674,19 +674,22 @@ __device__ __forceinline__ void grid_unit_paired(float2* smem, int q0, int V, in
 // (shfl.xor 16), so that each lane then holds all its first-pass inputs.
 // The taps of a quarter-warp (the unit in which 16-byte loads are served)
 // are those of 8 consecutive rows of one column, as in grid_unit_paired.
-// PS point pairs per gather step.
-template <int M, int TPL, int MAXR, int NC = 0, int PS = 2>
+// PS point pairs per gather step.  tid: the thread among the column pair's 2 TPL
+// (whole warps; -1: threadIdx.x); `sync` the barrier that covers them.
+template <int M, int TPL, int MAXR, int NC = 0, int PS = 2, class SYNC = BlockSync>
 __device__ __forceinline__ void grid_unit_xchg(float2* smem, int q, int V, int N, const float4* __restrict__ Z2,
                                                const int* __restrict__ gJ, const float2* __restrict__ gF,
-                                               float2* __restrict__ Tp, const float2* __restrict__ tw) {
+                                               float2* __restrict__ Tp, const float2* __restrict__ tw,
+                                               const SYNC& sync = SYNC(), int tid = -1) {
+    if (tid < 0) tid = threadIdx.x;
     constexpr int H = M >> 1;
     constexpr int PPL = M / TPL;   // first-pass inputs per thread (16, or 12 for lengths 3 * 2^a)
     constexpr int PPT = PPL / 2;   // point pairs gathered per thread
     static_assert(TPL % 16 == 0, "half-warps of 16 consecutive threads of a column");
     static_assert(PPL % 4 == 0 && PPT % PS == 0, "steps of the upper and lower half rows");
-    const int lane = threadIdx.x & 31;
-    const int h = lane >> 4;                                   // 0: column q, 1: column -q
-    const int t = ((threadIdx.x >> 5) << 4) + (lane & 15);     // thread index within the column
+    const int lane = tid & 31;
+    const int h = lane >> 4;                          // 0: column q, 1: column -q
+    const int t = ((tid >> 5) << 4) + (lane & 15);    // thread index within the column
     const bool live = q < H;
     const int* gJq = gJ + (size_t)(live ? q : 0) * M;
     const float2* gFq = gF + (size_t)(live ? q : 0) * M;
@@ -784,7 +787,7 @@ __device__ __forceinline__ void grid_unit_xchg(float2* smem, int q, int V, int N
     }
     // the origin (row 0 of column q = 0, input 0 of thread 0, the gather gave 0
     // there) is single-valued: mean over angles of the DC bin, by warp 0
-    if (live && q == 0 && threadIdx.x < 32) {
+    if (live && q == 0 && tid < 32) {
         float sx = 0.f, sy = 0.f;
         for (int j = lane; j < V; j += 32) {
             const float4 zz = __ldg(Z2 + paired_slot(j, 0, H, V));
@@ -800,7 +803,7 @@ __device__ __forceinline__ void grid_unit_xchg(float2* smem, int q, int V, int N
     }
     const SmemLine sm{smem + h * smem_line_len(M)};
     const ColDst<NC> dst{Tp, N, M, h == 0 ? q : (q == 0 ? H : M - q), h == 1 && q != 0, live};
-    fft_line_regs<M, TPL, true, MAXR>(t, x, dst, sm, tw);
+    fft_line_regs<M, TPL, true, MAXR>(t, x, dst, sm, tw, sync);
 }
 
 // row P6 + P7 + P8 for row tiles rb0 .. rb0 + TPC - 1 of RPT rows each (RPT TPL

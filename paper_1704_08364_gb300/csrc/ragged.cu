@@ -58,9 +58,16 @@ template <int M> __host__ __device__ constexpr int r_grid_pairs() { return RAGGE
 template <int M> __host__ __device__ constexpr int r_row_rpt() { return 4 * tpl_of<M>() <= RAGGED_WT ? 4 : 2; }
 template <int M> __host__ __device__ constexpr int r_row_tiles() { return RAGGED_WT / (r_row_rpt<M>() * tpl_of<M>()); }
 
+// two angle rows: interleaved over the lanes, as in the per-size kernel
+template <int M> __host__ __device__ constexpr bool r_ray_ilv() { return r_ray_lines<M>() == 2; }
+// threads that meet at one barrier within a unit of sets of `lines` lines
+template <int M> __host__ __device__ constexpr int r_group(int lines) {
+    return lines * tpl_of<M>() > 128 ? lines * tpl_of<M>() : 128;
+}
+
 // shared memory of one worker (float2 elements): the largest of its units
 template <int M> __host__ __device__ constexpr size_t r_worker_smem() {
-    const size_t a = (size_t)r_ray_lines<M>() * smem_line_len(M);
+    const size_t a = (size_t)r_ray_lines<M>() * ray_line_stride<M, r_ray_ilv<M>()>();
     const size_t b = (size_t)2 * r_grid_pairs<M>() * smem_line_len(M);
     const size_t c = (size_t)r_row_rpt<M>() * r_row_tiles<M>() * row_line_stride<M>();
     return a > b ? (a > c ? a : c) : (b > c ? b : c);
@@ -81,24 +88,38 @@ __host__ __device__ constexpr size_t r_max_worker_smem() {
 // kernel (inlining them all spills kilobytes).  NC = M/2 serves items of pad
 // factor 2 (N known at compile time: the first pass skips the zero padding and
 // the last the dropped outputs, as in the per-size kernels); NC = 0 the others.
+//
+// Within a unit, groups of r_group threads (whole lines, at least 128 threads)
+// work on lines of their own and meet at a barrier of their own, so that the
+// lines of the small lengths do not wait for each other between FFT passes.
 template <int M, int MAXR, int NC>
 __device__ __noinline__ void ray_u(float2* smem, const RItem& it, int u, const WorkerSync& sync, int tid) {
     constexpr int TPL = tpl_of<M>(), L = r_ray_lines<M>();
-    ray_unit<M, TPL, L, MAXR, NC, WorkerSync>(smem, u * L, it.V, it.N, it.sa, it.sb, BSTK_FILTER | BSTK_PAIRED, it.g,
-                                              it.two_alpha, it.Z, it.tw, sync, tid);
+    constexpr bool ILV = r_ray_ilv<M>();
+    constexpr int GT = r_group<M>(ILV ? 2 : 1), GL = GT / TPL;
+    const int g = tid / GT;
+    const WorkerSync gs = sync.group(g, GT);
+    ray_unit<M, TPL, GL, MAXR, NC, WorkerSync, ILV, true>(smem + g * GL * ray_line_stride<M, ILV>(), u * L + g * GL, it.V,
+                                                          it.N, it.sa, it.sb, BSTK_FILTER | BSTK_PAIRED, it.g,
+                                                          it.two_alpha, it.Z, it.tw, gs, tid % GT);
 }
 template <int M, int MAXR, int NC>
 __device__ __noinline__ void grid_u(float2* smem, const RItem& it, int u, const WorkerSync& sync, int tid) {
-    constexpr int TPL = tpl_of<M>(), CP = r_grid_pairs<M>();
-    grid_unit_paired<M, TPL, CP, MAXR, NC, 2, WorkerSync>(smem, u * CP, it.V, it.N,
-                                                          reinterpret_cast<const float4*>(it.Z), it.gJ, it.gF, it.T,
-                                                          it.tw, sync, tid);
+    constexpr int TPL = tpl_of<M>(), CP = r_grid_pairs<M>(), GT = r_group<M>(2);
+    const int c = tid / (2 * TPL);
+    const WorkerSync gs = sync.group(tid / GT, GT);
+    grid_unit_xchg<M, TPL, MAXR, NC, 1, WorkerSync>(smem + c * 2 * smem_line_len(M), u * CP + c, it.V, it.N,
+                                                    reinterpret_cast<const float4*>(it.Z), it.gJ, it.gF, it.T, it.tw,
+                                                    gs, tid % (2 * TPL));
 }
 template <int M, int MAXR, int NC>
 __device__ __noinline__ void row_u(float2* smem, const RItem& it, int u, const WorkerSync& sync, int tid) {
     constexpr int TPL = tpl_of<M>(), TT = r_row_tiles<M>(), RPT = r_row_rpt<M>();
-    row_unit<M, TPL, TT, MAXR, NC, WorkerSync, RPT>(smem, u * TT, it.N, it.T, it.va, it.vb, it.scale, it.tw,
-                                                    nullptr, sync, tid);
+    constexpr int GT = r_group<M>(RPT), GTT = GT / (RPT * TPL);
+    const int g = tid / GT;
+    const WorkerSync gs = sync.group(g, GT);
+    row_unit<M, TPL, GTT, MAXR, NC, WorkerSync, RPT>(smem + g * GTT * RPT * row_line_stride<M>(), u * TT + g * GTT, it.N,
+                                                     it.T, it.va, it.vb, it.scale, it.tw, nullptr, gs, tid % GT);
 }
 template <int M, int MAXR, int NC>
 __device__ __forceinline__ void run_unit_nc(float2* smem, const RItem& it, int stage, int u, const WorkerSync& sync,
@@ -127,7 +148,7 @@ __global__ void __launch_bounds__(RAGGED_THREADS, 1)
     __shared__ int s_u[RAGGED_WORKERS], s_ok[RAGGED_WORKERS];
     const int wk = threadIdx.x / RAGGED_WT;
     const int tid = threadIdx.x % RAGGED_WT;
-    const WorkerSync sync{1 + wk, RAGGED_WT};
+    const WorkerSync sync{1 + wk, RAGGED_WT};   // barriers 3 .. 10: groups of at least 128 of its threads
     float2* wsm = smem + (size_t)wk * r_max_worker_smem();
     int claimed = -1;   // thread 0: the entry claimed ahead of time
     for (;;) {
