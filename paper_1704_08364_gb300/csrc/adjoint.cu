@@ -133,7 +133,7 @@ struct ColOut {
 // Lane order: pair, then position, so that the stores of a warp are contiguous;
 // the pairs' lines are skewed by 32 / P banks.  Pairs beyond npairs are zero.
 template <int M, int P> __host__ __device__ constexpr int adj_col_stride() {
-    return smem_line_len(M) + (P > 1 ? 16 / P : 0);
+    return smem_line_len(M, P) + (P > 1 ? 16 / P : 0);
 }
 template <int M, int TPL, int LINES, int P>
 __global__ void __launch_bounds__(TPL * LINES)
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(TPL * LINES)
     const int c = blockIdx.x * (LINES / P) + cl;
     TileColSrc src{T + (size_t)pl * ((N + 3) / 4) * 4 * M, N, M, c, pl < npairs && c < M};
     ColOut dst{X + ((size_t)blockIdx.y * M + c) * M * P + p, P, c < M};
-    SmemLine sm{smem + (cl * P + p) * adj_col_stride<M, P>()};
+    LineOf<P> sm{smem + (cl * P + p) * adj_col_stride<M, P>()};
     fft_line<M, TPL, false>(t, src, dst, sm, tw);
 }
 
@@ -251,7 +251,7 @@ struct SinoCrop {
 // the next lane by a shuffle, across warps through `edge`).  Reading every cell
 // once per sample and pair instead (four times, 8 bytes of each 32-byte sector)
 // waited on the list-to-point chains (16 stall cycles per issue): 486 us for
-// the 8 pairs of 16 x 1024 x 1024, 280 us with this form and 212 us with the next
+// the 8 pairs of 16 x 1024 x 1024, 280 us with this form and 221 us with the next
 // cell's list bounds read ahead.  What bounds it
 // now is the latency and sector traffic of the point reads from L2.
 template <int M, int TPL, int LINES, int P>

@@ -289,17 +289,57 @@ struct WorkerSync {
 
 // ---- line storage ----------------------------------------------------------
 
-// Shared-memory line with one padding slot per 16 elements (bank-conflict free
-// for the strided stores of the early passes).
-__host__ __device__ constexpr int smem_line_len(int M) { return M + M / 16; }
+// Shared-memory line of M complex values with ADD padding slots after every PER
+// (the 16-byte-pair banks hold 16 values; a half-warp's 16 accesses should fall on
+// 16 different ones).  Plain lines, and the exchanges between the passes of the
+// lengths 2^a, have one slot per 16: the first pass stores at 17 t + s, the later
+// ones move by whole groups.  That padding does not suit lengths 3 * 2^a, whose
+// first pass stores at 12 t + s (three accesses a bank): see exchange_per.
+// (`lines`: see exchange_per; four and more take the longest padding)
+__host__ __device__ constexpr int smem_line_len(int M, int lines = 1) {
+    return M % 3 == 0 && lines >= 4 ? (M + M / 12 + 15) / 16 * 16 : M + M / 16;
+}
 
-struct SmemLine {
+template <int PER, int ADD> struct PadLine {
     float2* p;
     static constexpr bool kSmem = true;
-    static constexpr bool kPlain = true;   // load/store are exactly p[i + i/16]
-    __device__ __forceinline__ float2 load(int i) const { return p[i + (i >> 4)]; }
-    __device__ __forceinline__ void store(int i, float2 v) const { p[i + (i >> 4)] = v; }
+    static constexpr int kPer = PER, kAdd = ADD, kLines = 1;
+    static __host__ __device__ constexpr int at(int i) { return i + i / PER * ADD; }
+    __device__ __forceinline__ float2 load(int i) const { return p[at(i)]; }
+    __device__ __forceinline__ void store(int i, float2 v) const { p[at(i)] = v; }
 };
+using SmemLine = PadLine<16, 1>;
+// a line among LINES over whose threads the lanes of a warp alternate
+template <int LINES> struct LineOf : SmemLine {
+    static constexpr int kLines = LINES;
+};
+
+// Padding of the exchange after pass p of the transform, with the lanes of a warp
+// alternating over `lines` lines (the lines' starts 16 / lines slots apart, so that
+// 16 / lines consecutive threads of a line share a half-warp).
+//   2^a: one slot per 16.
+//   3 * 2^a, first pass of radix R0 (stores at R0 t + s, loads of consecutive
+//     elements): R0 = 3 needs none, 6 and 12 one per 48 / lines elements.
+//   3 * 2^a, then radix 16 (stores at 16 R0 (j / R0) + j % R0 + R0 s): R0 slots per
+//     16 R0, which puts consecutive j on consecutive banks.
+// In each of them the stores of a butterfly are a constant apart (with one slot per
+// 16 they were not for 3 * 2^a).  Wavefronts per half-warp store of the first pass at
+// M = 3072: 3 -> 1 with one line, 2 -> 1 with two or four.  15 x 1201 x 1536
+// backprojection 652 -> 627 us, 64 x 768 x 768 554 -> 532, 512 x 192 x 192 291 -> 260.
+__host__ __device__ constexpr int exchange_per(int M, int p, int MAXR, int lines) {
+    const int r0 = radix_of(M, 0, MAXR);
+    if (M % 3 != 0) return 16;
+    if (p == 0) return r0 == 3 ? M : (48 / lines > 12 ? 48 / lines : 12);
+    return p == 1 && radix_of(M, 1, MAXR) == 16 ? 16 * r0 : 16;
+}
+__host__ __device__ constexpr int exchange_add(int M, int p, int MAXR) {
+    const int r0 = radix_of(M, 0, MAXR);
+    if (M % 3 != 0) return 1;
+    if (p == 0) return r0 == 3 ? 0 : 1;
+    return p == 1 && radix_of(M, 1, MAXR) == 16 ? r0 : 1;
+}
+template <int M, int P, int MAXR, int LINES>
+using Exchange = PadLine<exchange_per(M, P, MAXR, LINES), exchange_add(M, P, MAXR)>;
 
 // ---- passes ----------------------------------------------------------------
 
@@ -325,10 +365,22 @@ __device__ __forceinline__ constexpr bool dst_drop_group(int lo, int hi) {
     return false;
 }
 
-// true for a plain SmemLine (no weighting or remapping in load/store)
-template <class T, class = void> struct plain_line_trait { static constexpr bool value = false; };
-template <class T> struct plain_line_trait<T, decltype(void(T::kPlain))> { static constexpr bool value = T::kPlain; };
-template <class T> __host__ __device__ constexpr bool is_plain_line() { return plain_line_trait<T>::value; }
+// true for a shared-memory line whose load and store are its padded elements
+template <class T, class = void> struct pad_line_trait { static constexpr bool value = false; };
+template <class T> struct pad_line_trait<T, decltype(void(T::kPer))> { static constexpr bool value = true; };
+template <class T> __host__ __device__ constexpr bool is_pad_line() { return pad_line_trait<T>::value; }
+// loads of a pass at j + s NB, stores at base + s NS, are a constant apart (0: not)
+template <class T, int NB> __host__ __device__ constexpr int pad_load_step() {
+    if constexpr (is_pad_line<T>()) return T::kAdd == 0 || NB % T::kPer == 0 ? T::at(NB) : 0;
+    return 0;
+}
+template <class T, int NS, int R> __host__ __device__ constexpr int pad_store_step() {
+    if constexpr (is_pad_line<T>()) {
+        if (T::kAdd == 0 || T::kPer % (NS * R) == 0) return NS;   // a butterfly stays in one group
+        if (NS % T::kPer == 0) return T::at(NS);
+    }
+    return 0;
+}
 
 // w[s] = tw[s * b] for s = 1..R-1 (b = k M / (NS R)): the powers of two of the
 // base root come from the table, the others are products of at most three
@@ -411,11 +463,11 @@ __device__ __forceinline__ void stockham_pass(int t, const Src& src, const Dst& 
     for (int it = 0; it < IT; ++it) {
         const int j = t + it * TPL;
         if ((NB % TPL) == 0 || j < NB) {
-            if constexpr (is_plain_line<Src>() && NB % 16 == 0) {
-                // padded index of j + s NB is (j + j/16) + s (NB + NB/16): one base, constant offsets
-                const float2* p = src.p + j + (j >> 4);
+            constexpr int LS = pad_load_step<Src, NB>();
+            if constexpr (LS > 0) {
+                const float2* p = src.p + Src::at(j);
 #pragma unroll
-                for (int s = 0; s < R; ++s) a[it][s] = p[s * (NB + NB / 16)];
+                for (int s = 0; s < R; ++s) a[it][s] = p[s * LS];
             } else {
 #pragma unroll
                 for (int s = 0; s < R; ++s)
@@ -445,11 +497,9 @@ __device__ __forceinline__ void stockham_pass(int t, const Src& src, const Dst& 
             }
             Dft<R, INV>::run(a[it]);
             const int base = (j / NS) * NS * R + k;
-            if constexpr (is_plain_line<Dst>() && (NS % 16 == 0 || (NS == 1 && 16 % R == 0))) {
-                // the R outputs base + s NS stay in one 16-group (NS = 1, base a multiple
-                // of R) or move by whole groups (NS a multiple of 16): constant offsets
-                float2* p = dst.p + base + (base >> 4);
-                constexpr int PS = NS == 1 ? 1 : NS + NS / 16;
+            constexpr int PS = pad_store_step<Dst, NS, R>();
+            if constexpr (PS > 0) {
+                float2* p = dst.p + Dst::at(base);
 #pragma unroll
                 for (int s = 0; s < R; ++s) p[s * PS] = a[it][s];
             } else {
@@ -466,38 +516,42 @@ __device__ __forceinline__ void stockham_pass(int t, const Src& src, const Dst& 
 // Run passes PIDX.. of the length-M transform.  Pass 0 reads `src`, the last
 // pass writes `dst`; the others go through the shared-memory line `sm`.  The last
 // pass runs as thread tl of the line sml (t, sm unless the maps change there).
+// LINES: lines over which the lanes alternate in pass 0.
 // Every thread that `sync` covers must call this (it contains barriers).
-template <int M, int TPL, bool INV, int MAXR, int PIDX, int NS, bool TWT, class Src, class Dst, class SYNC>
-__device__ __forceinline__ void fft_run(int t, const Src& src, const Dst& dst, const SmemLine& sm, int tl,
-                                        const SmemLine& sml, const float2* __restrict__ tw, const SYNC& sync) {
+template <int M, int TPL, bool INV, int MAXR, int PIDX, int NS, bool TWT, int LINES, class Src, class Dst, class SYNC>
+__device__ __forceinline__ void fft_run(int t, const Src& src, const Dst& dst, float2* sm, int tl, float2* sml,
+                                        const float2* __restrict__ tw, const SYNC& sync) {
     constexpr int R = radix_of(M, PIDX, MAXR);
     constexpr bool LAST = (NS * R == M);
     constexpr int TB = pass_tab_base(M, MAXR, PIDX);
+    using In = Exchange<M, PIDX == 0 ? 0 : PIDX - 1, MAXR, LINES>;
+    using Out = Exchange<M, PIDX, MAXR, LINES>;
+    static_assert(LAST || Out::at(M - 1) < smem_line_len(M, LINES), "the exchange fits the line");
     if constexpr (PIDX == 0) {
         if constexpr (LAST) {
             stockham_pass<M, R, NS, TPL, INV, TWT, TB>(t, src, dst, tw, Src::kSmem && Dst::kSmem, sync);
         } else {
-            stockham_pass<M, R, NS, TPL, INV, TWT, TB>(t, src, sm, tw, Src::kSmem, sync);
+            stockham_pass<M, R, NS, TPL, INV, TWT, TB>(t, src, Out{sm}, tw, Src::kSmem, sync);
             sync();
-            fft_run<M, TPL, INV, MAXR, PIDX + 1, NS * R, TWT>(t, src, dst, sm, tl, sml, tw, sync);
+            fft_run<M, TPL, INV, MAXR, PIDX + 1, NS * R, TWT, LINES>(t, src, dst, sm, tl, sml, tw, sync);
         }
     } else {
         if constexpr (LAST) {
-            stockham_pass<M, R, NS, TPL, INV, TWT, TB>(tl, sml, dst, tw, Dst::kSmem, sync);
+            stockham_pass<M, R, NS, TPL, INV, TWT, TB>(tl, In{sml}, dst, tw, Dst::kSmem, sync);
         } else {
-            stockham_pass<M, R, NS, TPL, INV, TWT, TB>(t, sm, sm, tw, true, sync);
+            stockham_pass<M, R, NS, TPL, INV, TWT, TB>(t, In{sm}, Out{sm}, tw, true, sync);
             sync();
-            fft_run<M, TPL, INV, MAXR, PIDX + 1, NS * R, TWT>(t, src, dst, sm, tl, sml, tw, sync);
+            fft_run<M, TPL, INV, MAXR, PIDX + 1, NS * R, TWT, LINES>(t, src, dst, sm, tl, sml, tw, sync);
         }
     }
 }
 
 // TWT: twiddles from the per-pass tables (one coalesced load each) instead of
 // four base-table loads and products per butterfly
-template <int M, int TPL, bool INV, int MAXR = 16, bool TWT = false, class Src, class Dst, class SYNC = BlockSync>
-__device__ __forceinline__ void fft_line(int t, const Src& src, const Dst& dst, const SmemLine& sm,
+template <int M, int TPL, bool INV, int MAXR = 16, bool TWT = false, class Src, class Dst, class SM, class SYNC = BlockSync>
+__device__ __forceinline__ void fft_line(int t, const Src& src, const Dst& dst, const SM& sm,
                                          const float2* __restrict__ tw, const SYNC& sync = SYNC()) {
-    fft_run<M, TPL, INV, MAXR, 0, 1, TWT>(t, src, dst, sm, t, sm, tw, sync);
+    fft_run<M, TPL, INV, MAXR, 0, 1, TWT, SM::kLines>(t, src, dst, sm.p, t, sm.p, tw, sync);
 }
 
 // Two thread-to-line maps for one transform: the first pass (LATE: all but the
@@ -510,18 +564,19 @@ __device__ __forceinline__ void fft_line(int t, const Src& src, const Dst& dst, 
 // threads of all the lines.  A transform of a single pass cannot change maps
 // (fft_remaps: then t0 = t1, sm0 = sm1).
 template <int M, int MAXR = 16> __host__ __device__ constexpr bool fft_remaps() { return radix_of(M, 0, MAXR) < M; }
-template <int M, int TPL, bool INV, int MAXR, bool TWT, bool LATE, class Src, class Dst, class SYNC = BlockSync>
-__device__ __forceinline__ void fft_line_remap(int t0, const Src& src, const SmemLine& sm0, int t1, const Dst& dst,
-                                               const SmemLine& sm1, const float2* __restrict__ tw,
+template <int M, int TPL, bool INV, int MAXR, bool TWT, bool LATE, class Src, class Dst, class SM0, class SM1,
+          class SYNC = BlockSync>
+__device__ __forceinline__ void fft_line_remap(int t0, const Src& src, const SM0& sm0, int t1, const Dst& dst,
+                                               const SM1& sm1, const float2* __restrict__ tw,
                                                const SYNC& sync = SYNC()) {
     constexpr int R = radix_of(M, 0, MAXR);
     static_assert(!Src::kSmem, "a source outside the lines");
     if constexpr (LATE || !fft_remaps<M, MAXR>()) {
-        fft_run<M, TPL, INV, MAXR, 0, 1, TWT>(t0, src, dst, sm0, t1, sm1, tw, sync);
+        fft_run<M, TPL, INV, MAXR, 0, 1, TWT, SM0::kLines>(t0, src, dst, sm0.p, t1, sm1.p, tw, sync);
     } else {
-        stockham_pass<M, R, 1, TPL, INV, TWT, 0>(t0, src, sm0, tw, false, sync);
+        stockham_pass<M, R, 1, TPL, INV, TWT, 0>(t0, src, Exchange<M, 0, MAXR, SM0::kLines>{sm0.p}, tw, false, sync);
         sync();
-        fft_run<M, TPL, INV, MAXR, 1, R, TWT>(t1, src, dst, sm1, t1, sm1, tw, sync);
+        fft_run<M, TPL, INV, MAXR, 1, R, TWT, SM0::kLines>(t1, src, dst, sm1.p, t1, sm1.p, tw, sync);
     }
 }
 
@@ -533,9 +588,9 @@ __device__ __forceinline__ void fft_line_remap(int t0, const Src& src, const Sme
 // passes are those of fft_line.  Call with every thread of the block; `sm`
 // must be free for writing (the caller's barrier).
 // sm1, t1: storage and thread of the later passes, as in fft_line_remap.
-template <int M, int TPL, bool INV, int MAXR = 16, class Dst, class SYNC = BlockSync, bool TWT = false>
-__device__ __forceinline__ void fft_line_regs(int t, float2 (&x)[M / TPL], const Dst& dst, const SmemLine& sm, int t1,
-                                              const SmemLine& sm1, const float2* __restrict__ tw,
+template <int M, int TPL, bool INV, int MAXR = 16, class Dst, class SYNC = BlockSync, bool TWT = false, class SM0, class SM1>
+__device__ __forceinline__ void fft_line_regs(int t, float2 (&x)[M / TPL], const Dst& dst, const SM0& sm, int t1,
+                                              const SM1& sm1, const float2* __restrict__ tw,
                                               const SYNC& sync = SYNC()) {
     constexpr int R = radix_of(M, 0, MAXR);
     constexpr int NB = M / R;
@@ -555,24 +610,19 @@ __device__ __forceinline__ void fft_line_regs(int t, float2 (&x)[M / TPL], const
 #pragma unroll
         for (int s = 0; s < R; ++s) a[s] = x[it + s * IT];
         Dft<R, INV>::run(a);
-        const int base = (t + it * TPL) * R;
-        if constexpr (16 % R == 0) {
-            // base is a multiple of R, so the R outputs stay in one 16-group
-            float2* p = sm.p + base + (base >> 4);
+        using Out = Exchange<M, 0, MAXR, SM0::kLines>;
+        static_assert(pad_store_step<Out, 1, R>() == 1, "a butterfly's outputs side by side");
+        float2* p = sm.p + Out::at((t + it * TPL) * R);
 #pragma unroll
-            for (int s = 0; s < R; ++s) p[s] = a[s];
-        } else {
-#pragma unroll
-            for (int s = 0; s < R; ++s) sm.store(base + s, a[s]);
-        }
+        for (int s = 0; s < R; ++s) p[s] = a[s];
     }
     if constexpr (R < M) {
         sync();
-        fft_run<M, TPL, INV, MAXR, 1, R, TWT>(t1, sm1, dst, sm1, t1, sm1, tw, sync);
+        fft_run<M, TPL, INV, MAXR, 1, R, TWT, SM0::kLines>(t1, sm1, dst, sm1.p, t1, sm1.p, tw, sync);
     }
 }
-template <int M, int TPL, bool INV, int MAXR = 16, class Dst, class SYNC = BlockSync, bool TWT = false>
-__device__ __forceinline__ void fft_line_regs(int t, float2 (&x)[M / TPL], const Dst& dst, const SmemLine& sm,
+template <int M, int TPL, bool INV, int MAXR = 16, class Dst, class SYNC = BlockSync, bool TWT = false, class SM>
+__device__ __forceinline__ void fft_line_regs(int t, float2 (&x)[M / TPL], const Dst& dst, const SM& sm,
                                               const float2* __restrict__ tw, const SYNC& sync = SYNC()) {
     fft_line_regs<M, TPL, INV, MAXR, Dst, SYNC, TWT>(t, x, dst, sm, t, sm, tw, sync);
 }

@@ -23,6 +23,8 @@
 //   k_grid_col_xchg  the same for one column pair per block with the first
 //               FFT pass of both columns fed from registers (partner lanes
 //               swap the halves of their gathered point pairs).
+//   (groups of 2 to 8 slice pairs take the three kernels of bst_inter.cuh instead,
+//   unless the plan's shape or the workspace's alignment rules them out.)
 //   k_row_ifft  the row half of P6 + P7 + P8: inverse FFT along c' for four
 //               rows at a time, keep the N central columns, scale by
 //               dt dw^2 = N / (2 M^2), write Re to slice a and Im to slice b.

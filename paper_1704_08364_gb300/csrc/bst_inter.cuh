@@ -34,7 +34,7 @@ template <int P> __host__ __device__ constexpr int inter_rows() { return 8 / P; 
 // pairs whose lines share a warp in the ray and row kernels (32-byte pieces)
 template <int P> __host__ __device__ constexpr int inter_lanes() { return P < 4 ? P : 4; }
 // stride between lines whose lanes alternate over n lines: skewed by 32 / n banks
-template <int M> __host__ __device__ constexpr int inter_stride(int n) { return smem_line_len(M) + 16 / n; }
+template <int M> __host__ __device__ constexpr int inter_stride(int n) { return smem_line_len(M, n) + 16 / n; }
 
 // Place of slot k, sign s (0: +k, 1: -k) in a row, in complex values: [k][s][P],
 // for P = 2 [k / 2][s][k % 2][P], so that the ray kernel writes whole sectors there
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(2 * inter_pairs<M>() * tpl_of<M>(), 1024 / (2 
         }
         __syncthreads();
     }
-    const SmemLine sm{smem + (e + P * w) * inter_stride<M>(P)};
+    const LineOf<P> sm{smem + (e + P * w) * inter_stride<M>(P)};
     const InterColDst<M, P, NC> dst{T + (size_t)grp * N * M * P + 2 * u + w, N,
                                     h == 0 ? q : (q == 0 ? H : M - q), h == 1 && q != 0};
     fft_line_regs<M, TPL, true, MAXR>(t, x, dst, sm, tw);
@@ -312,8 +312,8 @@ __global__ void __launch_bounds__(4 * tpl_of<M>() * inter_row_tiles<M>(), 1024 /
     const VolDst<NC> dst{vol + (size_t)sa * N * N + at, sb < slices ? vol + (size_t)sb * N * N + at : nullptr,
                          N, M, scale, r < N, nullptr};
     float2* base = smem + tile * 4 * row_line_stride<M>();
-    fft_line_remap<M, TPL, true, MAXR, false, true>(m.t0, src, SmemLine{base + m.line0 * row_line_stride<M>()}, m.t1, dst,
-                                       SmemLine{base + m.line1 * row_line_stride<M>()}, tw);
+    fft_line_remap<M, TPL, true, MAXR, false, true>(m.t0, src, LineOf<4>{base + m.line0 * row_line_stride<M>()}, m.t1, dst,
+                                                   SmemLine{base + m.line1 * row_line_stride<M>()}, tw);
 }
 
 }  // namespace bst

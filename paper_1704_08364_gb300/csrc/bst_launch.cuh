@@ -113,12 +113,12 @@ bst_status_t launch_forward_M(bst_plan_s* p, const float* sino, int slices, int 
     const float two_alpha = (float)(2 * p->alpha);
     const int row_tiles = (N + 3) / 4;
     const bool kbg = p->grid_kind == BST_GRID_KAISER_BESSEL;
-    if (kbg && mode != BSTK_RAW) mode |= BSTK_KBW;
+    if (kbg) mode |= BSTK_KBW;
     // The paired and interleaved layouts serve the bilinear gridding only; their
     // kernels read the workspace 16 bytes at a time, so a workspace that is not
     // so aligned takes the packed layout.  Groups of inter_pairs<M>() slice
     // pairs are interleaved; what remains of a chunk is paired.
-    const bool wide = !kbg && mode != BSTK_RAW && ((uintptr_t)ws & 15) == 0;
+    const bool wide = !kbg && ((uintptr_t)ws & 15) == 0;
     const bool paired = wide && p->fwd_layout != BST_LAYOUT_PACKED;
     const bool inter = wide && p->fwd_layout == BST_LAYOUT_INTERLEAVED && InterCfg<M>::OK;
     const int base_mode = mode;

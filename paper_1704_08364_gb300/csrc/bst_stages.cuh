@@ -83,13 +83,12 @@ __device__ __forceinline__ void spec_store(float2* z, int j, int V, int M, int m
 }
 
 // Weight W[|k|] of bin k for `mode` (times the polar cell area |k|, 1/4 at
-// k = 0, with BSTK_KBW); the Nyquist bin is zero unless the mode is raw.
+// k = 0, with BSTK_KBW); the Nyquist bin is zero.
 __device__ __forceinline__ float bin_weight(int k, int M, int mode, const float* __restrict__ g, float two_alpha) {
     const int ak = k <= (M >> 1) ? k : M - k;
     const int md = mode & 7;
     float w;
-    if (md == BSTK_RAW) w = 1.f;
-    else if (ak == (M >> 1)) w = 0.f;
+    if (ak == (M >> 1)) w = 0.f;
     else if (md == BSTK_FILTER) w = g ? __ldg(g + ak) : 1.f;
     else w = ak == 0 ? 0.f : __fdiv_rn(two_alpha, (float)ak);
     if (mode & BSTK_KBW) w *= ak == 0 ? 0.25f : (float)ak;
@@ -281,7 +280,8 @@ struct VolDst {
     }
 };
 
-template <int M> __host__ __device__ constexpr int row_line_stride() { return smem_line_len(M) + 4; }
+// stride of the RPT interleaved lines of a tile
+template <int M, int RPT = 4> __host__ __device__ constexpr int row_line_stride() { return smem_line_len(M, RPT) + 16 / RPT; }
 
 // ---- pre-reconstruction stages fused into the ray load and the weight ------
 //
@@ -825,9 +825,10 @@ __device__ __forceinline__ void row_unit(float2* smem, int rb0, int N, const flo
     const int rr = r1 < N ? r1 : 0;
     const VolDst<NC> dst{va + (size_t)rr * N, vb ? vb + (size_t)rr * N : nullptr, N, M,
                          dk ? scale * __ldg(dk + rr) : scale, r1 < N, dk};
-    float2* base = smem + tile * RPT * row_line_stride<M>();
-    fft_line_remap<M, TPL, true, MAXR, TWT, true>(m.t0, src, SmemLine{base + m.line0 * row_line_stride<M>()}, m.t1, dst,
-                                            SmemLine{base + m.line1 * row_line_stride<M>()}, tw, sync);
+    constexpr int LS = row_line_stride<M, RPT>();
+    float2* base = smem + tile * RPT * LS;
+    fft_line_remap<M, TPL, true, MAXR, TWT, true>(m.t0, src, LineOf<RPT>{base + m.line0 * LS}, m.t1, dst,
+                                                  SmemLine{base + m.line1 * LS}, tw, sync);
 }
 
 }  // namespace bst

@@ -69,7 +69,7 @@ template <int M> __host__ __device__ constexpr int r_group(int lines) {
 template <int M> __host__ __device__ constexpr size_t r_worker_smem() {
     const size_t a = (size_t)r_ray_lines<M>() * ray_line_stride<M, r_ray_ilv<M>()>();
     const size_t b = (size_t)2 * r_grid_pairs<M>() * smem_line_len(M);
-    const size_t c = (size_t)r_row_rpt<M>() * r_row_tiles<M>() * row_line_stride<M>();
+    const size_t c = (size_t)r_row_rpt<M>() * r_row_tiles<M>() * row_line_stride<M, r_row_rpt<M>()>();
     return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
 
@@ -118,7 +118,7 @@ __device__ __noinline__ void row_u(float2* smem, const RItem& it, int u, const W
     constexpr int GT = r_group<M>(RPT), GTT = GT / (RPT * TPL);
     const int g = tid / GT;
     const WorkerSync gs = sync.group(g, GT);
-    row_unit<M, TPL, GTT, MAXR, NC, WorkerSync, RPT>(smem + g * GTT * RPT * row_line_stride<M>(), u * TT + g * GTT, it.N,
+    row_unit<M, TPL, GTT, MAXR, NC, WorkerSync, RPT>(smem + g * GTT * RPT * row_line_stride<M, RPT>(), u * TT + g * GTT, it.N,
                                                      it.T, it.va, it.vb, it.scale, it.tw, nullptr, gs, tid % GT);
 }
 template <int M, int MAXR, int NC>
