@@ -407,8 +407,11 @@ __global__ void k_cell_keys(Geo geo, int M, int* __restrict__ key, float2* __res
 // never goes to HBM.  Writing Y and reducing it in a second kernel took 54 +
 // 118 us for 16 x 1024 x 1024 (64 blocks a pair walking the angles: 12 %
 // occupancy), 65 us in this form.  Fixed order: deterministic.
+// 512 threads an SM at least: with 1024 (64 registers) the sums and a butterfly do
+// not fit, and most lengths spill (training step of 16 x 768 x 768 584 -> 538 us, 16 x
+// 1024 x 1024 836 -> 830).
 template <int M, int TPL, int LPC>
-__global__ void __launch_bounds__(TPL * LPC, (TPL * LPC <= 1024) ? 1024 / (TPL * LPC) : 1)
+__global__ void __launch_bounds__(TPL * LPC, (TPL * LPC <= 512) ? 512 / (TPL * LPC) : 1)
     k_fg_ray(const float* __restrict__ sino, int slices, int pair0, int N, int V, const float2* __restrict__ lam,
              int add, float* __restrict__ part, const float2* __restrict__ tw) {
     extern __shared__ float2 smem[];
