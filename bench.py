@@ -97,7 +97,7 @@ STAGE_NAMES = {0: "k_ray_fft", 1: "k_grid_col", 2: "k_row_ifft", 3: "k_ss_filter
 
 # DRAM bytes (read + write) per launch of each forward kernel from one ncu
 # capture of the dram__bytes_read.sum and dram__bytes_write.sum counters on
-# the volume-2048 geometry (16 slices: one launch of 8 pairs each, cold cache), keyed by
+# the volume-2048 geometry (64 slices: launches of 16 pairs each, cold cache), keyed by
 # a SHA-256 over the kernels' device-code headers (the host launcher lives in
 # another file, so host-only edits keep the record) and by the launch shape
 # that the capture ran.  A record applies only while the device code hashes
@@ -107,11 +107,11 @@ KERNEL_SOURCES = ["paper_1704_08364_gb300/csrc/bst_forward.cuh", "paper_1704_083
                   "paper_1704_08364_gb300/csrc/bst_fft.cuh", "paper_1704_08364_gb300/csrc/bst_geo.cuh",
                   "paper_1704_08364_gb300/csrc/bst_inter.cuh"]
 CAPTURED_TRAFFIC = [
-    {"sha": "5182a6ef3146a9c4f464342e17da68624378eacd4d1d37d661da52193c60e7df",
+    {"sha": "d3cdc24865886ed514ee40f9873ec38424fe9e91bd668359db6b12d474fa5880",
      "rays": 2048, "pad": 2,
-     "shape": {"layout": "paired", "chunk_pairs": 8, "pair_fast": 1, "max_radix": 16, "grid_xchg": 1},
-     "bytes": {"k_ray_fft": 271184896 + 476406272, "k_grid_col": 629041664 + 486836480,
-               "k_row_ifft": 536912640 + 237447424}},
+     "shape": {"layout": "interleaved", "chunk_pairs": 16, "pair_fast": 1, "max_radix": 16, "grid_xchg": 1},
+     "bytes": {"k_ray_fft": 536972288 + 1018608896, "k_grid_col": 1148157440 + 1020544512,
+               "k_row_ifft": 1073816320 + 508776448}},
 ]
 
 

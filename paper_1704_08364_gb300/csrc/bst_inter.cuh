@@ -19,10 +19,10 @@
 // P = 256 / TPL (2 at M = 2048, 4 at 1024, 8 from 512 down) keeps a block at 512
 // threads, 2 P column lines in 70 KB of shared memory and two blocks an SM; M >=
 // 3072 takes P = 2 in one block of 1024 threads.
-// Measured, us a pair, paired -> interleaved: M = 1024 (512 x 512) ray 2.53 -> 1.62,
-// gridding 5.96 -> 4.33, row 1.94 -> 1.66; M = 2048 (1024 x 1024) ray 7.3 -> 6.3,
-// gridding 21.2 -> 18.8, row 6.2 -> 6.4; M = 4096 (2048 x 2048) ray 26.2 -> 26.9,
-// gridding 89.4 -> 84.2, row 26.2 -> 24.2.
+// Measured, us a pair, paired -> interleaved: M = 1024 (512 x 512) ray 2.53 -> 1.59,
+// gridding 5.96 -> 4.26, row 1.94 -> 1.53; M = 4096 (2048 x 2048) ray 26.2 -> 23.4,
+// gridding 89.4 -> 79.6, row 26.2 -> 26.5.  What bounds the gridding now is still the
+// latency of its taps and their L1 wavefronts.
 #pragma once
 #include "bst_stages.cuh"
 

@@ -295,8 +295,9 @@ template <int M, int RPT = 4> __host__ __device__ constexpr int row_line_stride(
 // two tables per call, and the ray kernel reads them.  Evaluating them per
 // output (a 64-bit modulo, two sincospif; I0 per sample) made the ray kernel
 // issue 65.0 M warp instructions a pair at 2048 x 2000 against 22.9 M without
-// the stages: 95.7 us a pair, 66.9 us with the tables, 50 us
-// with the rays requested before the first is used (prep_gather).
+// the stages: 95.7 us a pair, 66.9 us with the tables, 50 us with the rays
+// requested before the first is used (prep_gather), 44 us since the interleaved
+// spectrum is written in whole sectors.
 struct PrepArgs {
     const float* dark;    // [S][N] or null (0)
     const float* flat;    // [S][N] or null (input is already y)
