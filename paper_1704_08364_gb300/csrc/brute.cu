@@ -124,12 +124,15 @@ __device__ __forceinline__ void fma_slices(float2 (&acc)[H][2], float w, const f
 // shared-memory wavefronts on average with R = 4 against 16 for two reads per
 // pixel and slice.  A batch of angles with a value that is not finite reads the
 // two samples of each pixel instead (a zero weight would not hide it).  What
-// bounds it: FP32 issue and the shared-memory wavefronts, about alike.  At
-// 512 x 512, 512 angles, 16 slices: 1033 us for the form with one pixel a
-// thread, two 4-byte loads a slice and 103 warp instructions per 32 pixels,
-// angle and 8 slices; 632 us with this one.
+// bounds it: FP32 issue and the shared-memory wavefronts, about alike, and with
+// few blocks the chain of a batch: staging loads, barrier, sums.  The loads of a
+// warp for a whole batch are issued together, and the next batch's geometry with
+// them (six blocks of eight slices an SM leave the registers): 512 x 512, 512 angles, 16
+// slices 632 -> 555 us, 64 x 64, 300 angles, one slice 75 -> 57 us.  The form with
+// one pixel a thread, two 4-byte loads a slice and 103 warp instructions per 32
+// pixels, angle and 8 slices took 1033 us.
 template <int H, int R>
-__global__ void __launch_bounds__(32 * SS_WARPS, R > 1 ? 7 : 8)
+__global__ void __launch_bounds__(32 * SS_WARPS, H > 1 ? 6 : R > 1 ? 7 : 8)
     k_ss_bp(const float* __restrict__ y, int S, int V, int N, const double2* __restrict__ cs64,
             const float2* __restrict__ cs32, const float* __restrict__ wq, float* __restrict__ vol) {
     constexpr int W = ss_w<R>();
@@ -147,45 +150,69 @@ __global__ void __launch_bounds__(32 * SS_WARPS, R > 1 ? 7 : 8)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c0 = blockIdx.x * SS_TX, r0 = blockIdx.y * TY;
     const int s0 = blockIdx.z * (4 * H);
-    auto geometry = [&](int buf, int jb) {
+    // a batch's geometry by its first SS_AB threads: the loads, and what follows them
+    double2 cs;
+    float2 cf;
+    float wj;
+    auto geometry_load = [&](int jb) {
         const int j = jb + threadIdx.x;
-        if (threadIdx.x < SS_AB && j < V) {
-            const double2 cs = cs64[j];
+        const bool in = threadIdx.x < SS_AB && j < V;
+        cs = in ? cs64[j] : make_double2(0.0, 0.0);
+        cf = in ? cs32[j] : make_float2(0.f, 0.f);
+        wj = in ? wq[j] : 0.f;
+    };
+    auto geometry = [&](int buf, int jb) {
+        if (threadIdx.x < SS_AB && jb + (int)threadIdx.x < V) {
             const double fc = (double)(c0 + SS_TX / 2 - N / 2) * cs.x + (double)(r0 + TY / 2 - N / 2) * cs.y +
                               (double)(N / 2);
             const double mn = fc - (SS_TX / 2) * cs.x - (TY / 2) * cs.y + fmin(0.0, (SS_TX - 1) * cs.x);
             const int lo = (int)floor(mn) - 1, ic = (int)floor(fc);
-            const float2 cf = cs32[j];
-            ang[buf][threadIdx.x] = make_float4(cf.x, cf.y, (float)(fc - (double)ic), wq[j]);
+            ang[buf][threadIdx.x] = make_float4(cf.x, cf.y, (float)(fc - (double)ic), wj);
             // pixel R - 1 lies below 1 + (R - 1) sin t; one more for its second sample
             const int top = R == 1 ? 1 : 2 + (int)((float)(R - 1) * cf.y);
             pos[buf][threadIdx.x] = make_int2((ic - lo) | (top << 16), lo);
         }
     };
     const float fx = (float)(lane - SS_TX / 2), fy = (float)(warp * R - TY / 2);
+    geometry_load(0);
     geometry(0, 0);
     for (int jb = 0, buf = 0; jb < V; jb += SS_AB, buf ^= 1) {
         __syncthreads();   // this batch's geometry is there, the previous batch's samples are done with
         const int na = min(SS_AB, V - jb);
         bool odd = false;   // a staged value is not finite
-        for (int a = warp; a < na; a += SS_WARPS) {
-            const int lo = pos[buf][a].y;
-            const float w = ang[buf][a].w;
+        geometry_load(jb + SS_AB);
+        // all of the warp's loads of the batch are issued before the first is used
+        constexpr int NU = SS_AB / SS_WARPS, NI = (H * W + 31) / 32;
+        float v[NU][NI][4];
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            const int a = warp + u * SS_WARPS;
             const float* yj = y + (size_t)(jb + a) * N;
+            const int lo = a < na ? pos[buf][a].y : N;
 #pragma unroll
-            for (int it = lane; it < H * W; it += 32) {
-                const int h = it >= W, i = it - h * W;
-                const int g = lo + i;
-                float v[4] = {0.f, 0.f, 0.f, 0.f};
-                if (g >= 0 && g < N) {
+            for (int n = 0; n < NI; ++n) {
+                const int it = lane + 32 * n, h = it >= W, g = lo + it - h * W;
+                const bool in = it < H * W && g >= 0 && g < N;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int s = s0 + 4 * h + q;
-                        if (s < S) v[q] = __ldg(yj + (size_t)s * V * N + g) * w;
-                    }
+                for (int q = 0; q < 4; ++q) {
+                    const int s = s0 + 4 * h + q;
+                    v[u][n][q] = in && s < S ? __ldg(yj + (size_t)s * V * N + g) : 0.f;
                 }
-                seg[a][h][i] = make_float4(v[0], v[1], v[2], v[3]);
-                odd |= !(fabsf(v[0]) + fabsf(v[1]) + fabsf(v[2]) + fabsf(v[3]) < INFINITY);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            const int a = warp + u * SS_WARPS;
+            if (a >= na) break;
+            const float w = ang[buf][a].w;
+#pragma unroll
+            for (int n = 0; n < NI; ++n) {
+                const int it = lane + 32 * n, h = it >= W, i = it - h * W;
+                if (it < H * W) {
+                    const float4 z = make_float4(v[u][n][0] * w, v[u][n][1] * w, v[u][n][2] * w, v[u][n][3] * w);
+                    seg[a][h][i] = z;
+                    odd |= !(fabsf(z.x) + fabsf(z.y) + fabsf(z.z) + fabsf(z.w) < INFINITY);
+                }
             }
         }
         geometry(buf ^ 1, jb + SS_AB);
@@ -322,18 +349,23 @@ bst_status_t bst_launch_brute(bst_plan_s* p, const float* sino, int slices, cons
         if (s != BST_OK) return s;
         y = q;
     }
-    // Four pixels a thread where that still gives every SM a few blocks; one
-    // pixel a thread (four times the blocks) where it does not, and four slices
-    // a thread where there are no more.
-    const long long blocks4 = (long long)((p->N + 31) / 32) * ((p->N + 15) / 16) * ((slices + 7) / 8);
+    // Slices and pixels a thread, by the blocks per SM that each shape gives.  Eight
+    // slices (four pixels) read a window for twice the slices, but a block takes
+    // 7/4 of the time of one of four slices, and below three blocks an SM its longer
+    // chain shows.  With four slices, more pixels a thread do less work in all, and
+    // fewer have the shorter chain.  300 angles, us with one, two, four pixels: 64 x 64
+    // 57, 61, 77; 16 slices of 192 x 192 130, 89, 91; 5 of 384 x 384 228, 165, 126;
+    // four and eight slices: 20 of 512 x 512 467, 494; 40 904, 754.
+    const auto blocks = [&](int h, int r) {
+        return (long long)((p->N + 31) / 32) * ((p->N + 4 * r - 1) / (4 * r)) * ((slices + 4 * h - 1) / (4 * h));
+    };
+    constexpr long long SMS = 152;
+    const long long b4 = blocks(1, 4), c4 = (b4 + SMS - 1) / SMS, c8 = (blocks(2, 4) + SMS - 1) / SMS;
     bst_timing_mark(p, st, -1);
-    if (slices > 4) {
-        if (blocks4 >= 304) bst::launch_ss_bp<2, 4>(p, y, slices, vol, st);
-        else bst::launch_ss_bp<2, 1>(p, y, slices, vol, st);
-    } else {
-        if (blocks4 >= 304) bst::launch_ss_bp<1, 4>(p, y, slices, vol, st);
-        else bst::launch_ss_bp<1, 1>(p, y, slices, vol, st);
-    }
+    if (c8 >= 3 && 7 * c8 < 4 * c4) bst::launch_ss_bp<2, 4>(p, y, slices, vol, st);
+    else if (5 * b4 > 12 * SMS) bst::launch_ss_bp<1, 4>(p, y, slices, vol, st);
+    else if (blocks(1, 1) > SMS) bst::launch_ss_bp<1, 2>(p, y, slices, vol, st);
+    else bst::launch_ss_bp<1, 1>(p, y, slices, vol, st);
     bst_timing_mark(p, st, 4);
     return cudaGetLastError() == cudaSuccess ? BST_OK : BST_ERR_CUDA;
 }
