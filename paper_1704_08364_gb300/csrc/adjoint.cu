@@ -46,13 +46,23 @@ template <int M, int P> __host__ __device__ constexpr int adj_col_lines() {
     return n > 1 ? n * P : P;
 }
 // lines (angle rows times P pairs) of a block of the polar kernel: its threads
-// walk the rows one after the other, so four rows at most (more only to fill a
-// warp)
+// walk the rows one after the other, so four rows at most, two with few pairs (more
+// only to fill a warp)
 template <int M, int P> __host__ __device__ constexpr int adj_polar_lines() {
-    const int warp = 32 / (adj_tpl<M>() * P), n = 256 / (adj_tpl<M>() * P);
-    const int rows = n > 4 ? 4 : n;
+    const int warp = 32 / (adj_tpl<M>() * P), n = 256 / (adj_tpl<M>() * P), most = P < 4 ? 2 : 4;
+    const int rows = n > most ? most : n;
     const int l = warp > rows ? warp : rows;
     return l > 1 ? l * P : P;
+}
+// threads of a block of the polar kernel: those of the lines' transforms, and up to
+// M = 1024 with few pairs as many again as a row has bins, 512 at most: one pair
+// alone fills the chip only so, and its walk is a chain of M (1 + 1 / rows) / threads
+// steps (one slice of 64 x 64 30.7 -> 19.8 us; 33 x 400 x 512, whose last pair is alone,
+// 204 -> 188).  From M = 1536 a pair has blocks enough (one slice of 900 x 1024 69.7 ->
+// 74.0 us with them).
+template <int M, int P> __host__ __device__ constexpr int adj_polar_threads() {
+    const int fft = adj_tpl<M>() * adj_polar_lines<M, P>(), most = M < 512 ? M : 512;
+    return M <= 1024 && P < 4 && most > fft ? most / fft * fft : fft;
 }
 
 // ---------------------------------------------------------------------------
@@ -259,14 +269,14 @@ struct SinoCrop {
 // the 8 pairs of 16 x 1024 x 1024, 280 us with this form and 221 us with the next
 // cell's list bounds read ahead.  What bounds it
 // now is the latency and sector traffic of the point reads from L2.
-template <int M, int TPL, int LINES, int P>
-__global__ void __launch_bounds__(TPL * LINES, 1024 / (TPL * LINES))
+template <int M, int TPL, int LINES, int P, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT)
     k_adj_polar(const float2* __restrict__ X, Cells cl, int V, int N, int slices, int pair0, int npairs, int mode,
                 const float* __restrict__ g, float two_alpha, float scale, float* __restrict__ sino,
                 float2* __restrict__ lam, const float2* __restrict__ tw) {
-    constexpr int NT = TPL * LINES, L = LINES / P, H = M / 2;
+    constexpr int L = LINES / P, H = M / 2;
     constexpr int EDGES = (M - 1) / 32;   // warp boundaries within a row
-    static_assert(NT % 32 == 0 && LINES % P == 0, "whole warps, whole groups of pairs");
+    static_assert(NT % 32 == 0 && TPL * LINES % 32 == 0 && LINES % P == 0, "whole warps, whole groups of pairs");
     extern __shared__ float2 smem[];
     __shared__ float2 edge[EDGES > 0 ? EDGES : 1][LINES];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -354,6 +364,8 @@ __global__ void __launch_bounds__(TPL * LINES, 1024 / (TPL * LINES))
         *q = cadd(*q, edge[w][line]);
     }
     __syncthreads();
+    if (tid >= TPL * LINES) return;   // the transforms' threads go on, with a barrier of their own
+    const WorkerSync sync{1, TPL * LINES};
     const int line = tid / TPL, t = tid % TPL, p = line % P;
     const int pl = blockIdx.y * P + p, j = j0 + line / P;
     const bool live = j < V && pl < npairs;
@@ -373,7 +385,7 @@ __global__ void __launch_bounds__(TPL * LINES, 1024 / (TPL * LINES))
     const int sa = 2 * (pair0 + pl), sb = sa + 1;
     SinoCrop dst{sino + ((size_t)sa * V + j) * N, sb < slices ? sino + ((size_t)sb * V + j) * N : nullptr, N, M,
                  scale, live};
-    fft_line<M, TPL, true>(t, src, dst, sm, tw);
+    fft_line<M, TPL, true>(t, src, dst, sm, tw, sync);
 }
 
 // ---------------------------------------------------------------------------
@@ -563,7 +575,8 @@ static void adjoint_group(bst_plan_s* p, const AdjLayout& L, int stage, int slic
     const Cells cl{p->cell_start, p->cell_pts, p->cell_w};
     const float scale = (float)((double)N / (2.0 * (double)M * (double)M));
     constexpr int LP = C::template LP<P>, LR = LP / P;
-    k_adj_polar<M, C::TPL, LP, P><<<dim3((V + LR - 1) / LR, groups), C::TPL * LP, C::template SP<P>, st>>>(
+    constexpr int NT = adj_polar_threads<M, P>();
+    k_adj_polar<M, C::TPL, LP, P, NT><<<dim3((V + LR - 1) / LR, groups), NT, C::template SP<P>, st>>>(
         X, cl, V, N, slices, p0 + at, np, mode, g, (float)(2 * p->alpha), scale, sino,
         keep_lam ? L.lam + (size_t)at * V * M : nullptr, p->tw);
     bst_timing_mark(p, st, 7);
@@ -573,7 +586,7 @@ template <int M, int P>
 static bool adjoint_smem() {
     using C = AdjCfg<M>;
     return set_smem_a(k_adj_col_fft<M, C::TPL, C::template LC<P>, P>, C::template SC<P>) &&
-           set_smem_a(k_adj_polar<M, C::TPL, C::template LP<P>, P>, C::template SP<P>);
+           set_smem_a(k_adj_polar<M, C::TPL, C::template LP<P>, P, adj_polar_threads<M, P>()>, C::template SP<P>);
 }
 
 template <int M>
