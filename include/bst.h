@@ -73,8 +73,8 @@ typedef enum {
     BST_LAYOUT_PAIRED = 1,  /* Z[V][M/2] pairs (Z[k], Z[-k]): one 16-byte load serves a
                                Cartesian point and its mirror (bilinear gridding only) */
     BST_LAYOUT_INTERLEAVED = 2  /* groups of 2 to 8 slice pairs interleaved point by point
-                               (FFT lengths from 32); pairs that fill no group take the
-                               paired layout */
+                               (FFT lengths from 32); pairs that fill no group, and
+                               small calls that have such pairs, take the paired layout */
 } bst_layout_t;
 
 /* Launch shape of the forward path (extension; no passage: the paper fixes

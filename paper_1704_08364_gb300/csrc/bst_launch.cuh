@@ -117,10 +117,14 @@ bst_status_t launch_forward_M(bst_plan_s* p, const float* sino, int slices, int 
     // The paired and interleaved layouts serve the bilinear gridding only; their
     // kernels read the workspace 16 bytes at a time, so a workspace that is not
     // so aligned takes the packed layout.  Groups of inter_pairs<M>() slice
-    // pairs are interleaved; what remains of a chunk is paired.
+    // pairs are interleaved; what remains of a chunk is paired.  A call with pairs
+    // left over is paired altogether below pairs M (V + N) = 2^23: three more launches
+    // cost it more than the groups save (12 pairs of 64 x 64 22.2 against 13.4 us, 6 of
+    // 512 x 512 59.5 against 50.8; 9 of 512 x 512, just above, 68.8 against 80.5).
     const bool wide = !kbg && ((uintptr_t)ws & 15) == 0;
     const bool paired = wide && p->fwd_layout != BST_LAYOUT_PACKED;
-    const bool inter = wide && p->fwd_layout == BST_LAYOUT_INTERLEAVED && InterCfg<M>::OK;
+    const bool inter = wide && p->fwd_layout == BST_LAYOUT_INTERLEAVED && InterCfg<M>::OK &&
+                       (pairs % bsth::inter_pairs_of(M) == 0 || (long long)pairs * M * (V + N) >= 1 << 23);
     const int base_mode = mode;
     if (paired) mode |= BSTK_PAIRED;
     const int pf = p->pair_fast ? 1 : 0;

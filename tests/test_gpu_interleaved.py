@@ -86,3 +86,22 @@ def test_workspace_aligned_to_eight_bytes(bst, N, S):
     st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     assert _lib.load().bst_fbp(plan.handle, p(d), S, None, p(out), p(ws, 8), nb, st) == 0
     assert_parity(out.cpu().numpy(), np.stack([ob.fbp(s.astype(np.float64), theta) for s in sino]), what=f"N={N}")
+
+
+@pytest.mark.parametrize("N,V,alpha,S", [(128, 60, 2, 349), (64, 50, 2, 1150), (384, 40, 2, 53), (768, 24, 2, 13)])
+def test_groups_and_pairs_left_over(bst, N, V, alpha, S):
+    """Calls large enough for groups although pairs are left over, and slices of
+    every kind of them (first group, last group, left over) against the oracle."""
+    M, pairs = alpha * N, (S + 1) // 2
+    assert pairs * M * (V + N) >= 1 << 23 and pairs % (8 if M <= 512 else 4 if M <= 1024 else 2)
+    rng = np.random.default_rng(N + S)
+    theta = synth.uniform_angles(V)
+    sino = rng.standard_normal((S, V, N)).astype(np.float32)
+    plan = bst.Plan(N, theta, alpha)
+    plan.set_forward_config(layout="interleaved", chunk_pairs=256)
+    got = plan.fbp(_cuda(sino)).cpu().numpy()
+    for s in (0, 7, S // 2, S - 18, S - 3, S - 2, S - 1):
+        if s >= 0:
+            assert_parity(got[s], ob.fbp(sino[s].astype(np.float64), theta, alpha), what=f"N={N} slice {s} of {S}")
+    plan.set_forward_config(layout="paired")
+    assert_parity(got, plan.fbp(_cuda(sino)).cpu().numpy(), what=f"N={N} paired")
