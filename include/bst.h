@@ -113,8 +113,9 @@ bst_status_t bst_plan_destroy(bst_plan_t plan);
  * slices (extension; no passage -- the memory budget of Sec. 4 bounds what a
  * GPU holds at once; here the caller allocates it): the padded polar
  * spectrum Z[chunk][V][M] and the column-transformed
- * grid T[chunk][N][M] (complex64) for a chunk of slice pairs sized to stay
- * resident in L2 where possible.  0 for an invalid plan or slices <= 0. */
+ * grid T[chunk][N][M] (complex64) for a chunk of slice pairs, twice where two
+ * chunks are in flight (chunk_pairs and max_lanes of bst_fwd_config_t set how
+ * much).  0 for an invalid plan or slices <= 0. */
 size_t bst_workspace_bytes(bst_plan_t plan, int slices);
 
 /* BST filtered backprojection (Sec. 2 stages P0..P8 with the FBP weight
@@ -305,8 +306,9 @@ bst_status_t bst_plan_get_gridding(bst_plan_t plan, int* kind, int* width);
  * or 2) and changes nothing on error; bst_workspace_bytes follows the new
  * chunk and lane counts, so size workspaces after setting it.  A plan starts
  * with radix 16, the interleaved layout, grid_xchg 1, chunks of about 64 MiB of
- * workspace but at least 8 pairs, block order pair-fastest from M = 2048 on,
- * and two lanes.  A workspace that is not 16-byte aligned takes the packed
+ * workspace but at least 8 pairs (fewer, down to one, where the workspace would
+ * exceed 4 GiB or a sixteenth of the device memory free at the plan's creation),
+ * block order pair-fastest from M = 2048 on, and two lanes.  A workspace that is not 16-byte aligned takes the packed
  * layout whatever the field says.  A Kaiser-Bessel plan
  * always uses the packed layout.  Errors: INVALID_ARGUMENT. */
 bst_status_t bst_plan_set_forward_config(bst_plan_t plan, const bst_fwd_config_t* config);

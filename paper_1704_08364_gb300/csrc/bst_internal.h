@@ -45,7 +45,8 @@ struct bst_plan_s {
     size_t kb_n = 0;
     int kb_nstrips = 0;
     int chunk_pairs = 1;            // slice pairs per chunk of the forward path
-    int chunk_default = 1;          // the chunk sized to about 64 MiB of workspace
+    int chunk_default = 1;          // the chunk that the plan started with (bsth::default_chunk)
+    size_t ws_most = 0;             // bytes of a workspace that more than one pair a lane may take
     int maxr = 16;                  // FFT radix schedule of the forward path (16 or 8; autotuned)
     int fwd_layout = 0;             // BST_LAYOUT_PACKED or BST_LAYOUT_PAIRED (autotuned)
     int pair_fast = 0;              // gridding blocks ordered pair-fastest (autotuned)
@@ -143,6 +144,23 @@ __host__ __device__ constexpr int inter_pairs_of(int M) {
     const int tpl = M % 3 == 0 ? M / 12 : M / 16;
     const int c = 256 / tpl > 8 ? 8 : tpl >= 256 ? 2 : 256 / tpl;
     return c > 0 && tpl % (16 / c) == 0 ? c : 1;
+}
+
+// Bytes that the forward workspace of a plan may take with more than one slice pair a
+// lane: 4 GiB, less where little device memory is free at the plan's creation.
+inline size_t workspace_most(size_t free_bytes) { return std::min<size_t>((size_t)4 << 30, free_bytes / 16); }
+
+// Slice pairs per chunk that a plan starts with: 64 MiB of workspace, but at least 8
+// pairs (whole groups), which fill several waves of blocks at every length; fewer,
+// down to one, where two lanes of them would take more than `most` bytes.  Chunks
+// of 2, 4, 8, 16 pairs: 64 x 2048 x 2048 4421, 4354, 4299, 4258 us; 512 x 512 x 512
+// 2360, 1751, 1656, 1651 us.  8 pairs of 2048 x 2048 at pad factor 2 take 2 GiB.
+inline int default_chunk(int M, size_t per_pair, size_t most) {
+    const size_t fit = std::min<size_t>(256, ((size_t)64 << 20) / per_pair);
+    const size_t want = std::max<size_t>(8, fit & ~(size_t)7), cap = most / (kMaxLanes * per_pair);
+    if (cap >= want) return (int)want;
+    const size_t g = (size_t)inter_pairs_of(M);
+    return (int)std::max<size_t>(1, cap >= g ? cap / g * g : cap);
 }
 
 // Slice pairs per chunk for a call of `pairs` pairs with at most `most` a chunk.

@@ -217,16 +217,17 @@ bst_status_t bst_plan_create(bst_plan_t* out, int rays, int angles, const float*
             return gs;
         }
     }
-    // The launch shape a plan starts with: interleaved groups, chunks of 64 MiB
-    // of workspace but at least 8 pairs (whole groups), which fill several waves
-    // of blocks at every length; pair-fastest gridding where a geometry table (6
-    // M^2 bytes) is too large to stay in L2 beside Z.  Against the packed layout
-    // with chunks of 64 MiB: 15 x 1201 x 1536 backprojection 1220 -> 815 us.
-    // Chunks of 2, 4, 8, 16 pairs: 64 x 2048 x 2048 4421, 4354, 4299, 4258 us; 512 x
-    // 512 x 512 2360, 1751, 1656, 1651 us.
-    const size_t budget = (size_t)64 << 20;
-    const size_t fit = std::min<size_t>(256, budget / bsth::fwd_bytes_per_pair(p));
-    p->chunk_pairs = (int)std::max<size_t>(8, fit & ~(size_t)7);
+    // The launch shape a plan starts with: interleaved groups; pair-fastest gridding
+    // where a geometry table (6 M^2 bytes) is too large to stay in L2 beside Z.
+    // Against the packed layout with chunks of 64 MiB: 15 x 1201 x 1536
+    // backprojection 1220 -> 815 us.
+    size_t free_bytes = 0, total_bytes = 0;
+    if (cudaMemGetInfo(&free_bytes, &total_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        free_bytes = ~(size_t)0;
+    }
+    p->ws_most = bsth::workspace_most(free_bytes);
+    p->chunk_pairs = bsth::default_chunk(M, bsth::fwd_bytes_per_pair(p), p->ws_most);
     p->fwd_layout = BST_LAYOUT_INTERLEAVED;
     p->grid_xchg = 1;
     p->pair_fast = M >= 2048;
