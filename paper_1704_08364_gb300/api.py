@@ -94,6 +94,19 @@ class Plan:
             self._ws[key] = buf
         return buf
 
+    def _chunked_workspace(self, kind: str, size, slices: int, device) -> torch.Tensor:
+        """The workspace of a chunked forward call, size(handle, slices) bytes.  Where
+        it cannot be allocated the plan goes on with chunks of half as many pairs,
+        down to one pair, the least that the path takes."""
+        while True:
+            try:
+                return self.workspace(kind, size(self._h, slices), device)
+            except torch.OutOfMemoryError:
+                pairs = min(self.forward_config["chunk_pairs"], (slices + 1) // 2)
+                if pairs <= 1:
+                    raise
+                self.set_forward_config(chunk_pairs=pairs // 2)
+
     def workspace_bytes(self, slices: int) -> int:
         return int(self._lib.bst_workspace_bytes(self._h, int(slices)))
 
@@ -208,7 +221,7 @@ class Plan:
         if g is not None:
             _need(g, "g", (self.M // 2,))
         out = self._volume(out, S, sino)
-        ws = self.workspace("fwd", self._lib.bst_workspace_bytes(self._h, S), sino.device)
+        ws = self._chunked_workspace("fwd", self._lib.bst_workspace_bytes, S, sino.device)
         if mode == FILTER:
             code = self._lib.bst_fbp(self._h, _ptr(sino), S, _ptr(g), _ptr(out), _ptr(ws), ws.numel(), _stream())
             _check(code, "bst_fbp")
@@ -237,7 +250,7 @@ class Plan:
         if out is None:
             out = torch.empty((S, self.rays, self.rays), dtype=torch.float32, device=sino.device)
         _need(out, "out", (S, self.rays, self.rays))
-        ws = self.workspace("fwd", self.workspace_bytes(S), sino.device)
+        ws = self._chunked_workspace("fwd", self._lib.bst_workspace_bytes, S, sino.device)
         _check(self._lib.bst_fbp_prep(self._h, _ptr(sino), S, _ptr(dark), _ptr(flat), float(shift), float(kb_beta),
                                       float(kb_halfwidth), _ptr(g), _ptr(out), _ptr(ws), ws.numel(), _stream()),
                "bst_fbp_prep")
@@ -277,8 +290,7 @@ class Plan:
         if g is not None:
             _need(g, "g", (self.M // 2,))
         dev = device or torch.device("cuda", torch.cuda.current_device())
-        nb = int(self._lib.bst_host_workspace_bytes(self._h, S))
-        ws = self.workspace("host", nb, dev)
+        ws = self._chunked_workspace("host", self._lib.bst_host_workspace_bytes, S, dev)
         _check(self._lib.bst_fbp_host(self._h, _ptr(sino), S, _ptr(g), _ptr(out), _ptr(ws), ws.numel(), _stream()),
                "bst_fbp_host")
         torch.cuda.current_stream().synchronize()
