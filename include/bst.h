@@ -315,13 +315,15 @@ bst_status_t bst_plan_set_forward_config(bst_plan_t plan, const bst_fwd_config_t
 bst_status_t bst_plan_get_forward_config(bst_plan_t plan, bst_fwd_config_t* config);
 
 /* Autotuner (extension; no passage): time the plan's forward path on a
- * synthetic batch of about 256 MiB (`slices` slices, at least two chunks of the
- * largest candidate; <= 0 picks that size) under each candidate launch shape --
- * radix 16 or 8; interleaved or paired layout (bilinear plans); half the plan's
- * default chunk, the default and twice it; either block order -- keep the fastest
- * (the best of three timed runs each, after one warm-up run) and return its
- * radix in *chosen (may be NULL).  Allocates and frees its own buffers;
- * synchronises the device. */
+ * synthetic batch of about 256 MiB (`slices` slices, at least one chunk of the
+ * largest candidate on each lane; <= 0 picks that size) under each candidate launch
+ * shape -- radix 16; interleaved or paired layout (bilinear plans); half the chunk
+ * that the plan started with, that chunk and twice it; either block order -- and
+ * keep the fastest (the best of three timed runs each, after one warm-up run)
+ * in place of the plan's present shape, which is not timed unless it is one of
+ * them.  Returns the radix in *chosen (may be NULL).  Allocates and frees its own
+ * buffers, at most half of the free device memory where it can: then it takes
+ * fewer slices, and leaves out the larger chunks.  Synchronises the device. */
 bst_status_t bst_plan_autotune(bst_plan_t plan, int slices, int* chosen);
 
 /* ---- ragged batch: sinograms of mixed sizes in one persistent launch ----- */

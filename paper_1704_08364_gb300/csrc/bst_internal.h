@@ -181,6 +181,71 @@ inline size_t prep_table_bytes(const bst_plan_s* p) {
     return ((size_t)p->M * sizeof(float2) + (size_t)p->N * sizeof(float) + 255) & ~(size_t)255;
 }
 
+// bytes of the forward workspace for `slices` slices in chunks of at most `most` pairs
+inline size_t fwd_ws_bytes(const bst_plan_s* p, int slices, int most) {
+    const int pairs = (slices + 1) / 2;
+    const int chunk = fwd_chunk(p, pairs, most);
+    const int nchunks = (pairs + chunk - 1) / chunk;
+    const int lanes = std::min(std::min(nchunks, kMaxLanes), std::max(p->max_lanes, 1));   // chunks in flight
+    return (size_t)lanes * chunk * fwd_bytes_per_pair(p) + prep_table_bytes(p);
+}
+
+// The candidate launch shapes of the autotuner, largest chunk first: for bilinear
+// plans the interleaved layout (where the length has it) and the paired one; twice
+// the default chunk, the default and half of it (a larger chunk fills more waves of
+// blocks, a smaller one keeps the intermediates in L2); either block order.  The
+// lane count stays the plan's.  Radix 8 (never fewer passes), the packed layout
+// and the paired gather through shared memory measured slower at every length
+// and are left to bst_plan_set_forward_config.
+inline std::vector<bst_fwd_config_t> tune_candidates(const bst_plan_s* p) {
+    std::vector<bst_fwd_config_t> out;
+    std::vector<int> layouts;
+    if (p->grid_kind != BST_GRID_BILINEAR) {
+        layouts = {BST_LAYOUT_PACKED};
+    } else {
+        if (inter_pairs_of(p->M) > 1) layouts.push_back(BST_LAYOUT_INTERLEAVED);
+        layouts.push_back(BST_LAYOUT_PAIRED);
+    }
+    int last = 0;
+    for (int ch : {std::min(256, 2 * p->chunk_default), p->chunk_default, std::max(1, p->chunk_default / 2)}) {
+        if (ch == last) continue;
+        last = ch;
+        for (int l : layouts)
+            for (int pf : {0, 1}) out.push_back(bst_fwd_config_t{16, l, ch, pf, p->max_lanes, 1});
+    }
+    return out;
+}
+
+// What the autotuner runs, within `room` bytes where it can: every candidate on
+// `slices` slices, but at least one chunk of the largest on each lane.  Where that
+// is too much, fewer slices, then without the largest chunks, and with the smallest
+// chunk alone as few slices as one pair.
+struct TuneRun {
+    std::vector<bst_fwd_config_t> shapes;
+    int slices = 0;
+    size_t ws = 0;      // workspace of the largest candidate
+};
+inline TuneRun tune_run(const bst_plan_s* p, int slices, size_t room) {
+    const size_t per_slice = ((size_t)p->V * p->N + (size_t)p->N * p->N) * sizeof(float);
+    TuneRun r;
+    r.shapes = tune_candidates(p);
+    for (;;) {
+        const int most = r.shapes.front().chunk_pairs;
+        const bool last = r.shapes.back().chunk_pairs == most;
+        const int least = last ? 2 : 2 * kMaxLanes * most;
+        for (r.slices = std::max(slices, 2 * kMaxLanes * most);; r.slices = std::max(least, r.slices / 2)) {
+            r.ws = 0;
+            for (const bst_fwd_config_t& c : r.shapes) r.ws = std::max(r.ws, fwd_ws_bytes(p, r.slices, c.chunk_pairs));
+            if (r.ws + r.slices * per_slice <= room) return r;
+            if (r.slices == least) break;
+        }
+        if (last) return r;
+        r.shapes.erase(std::remove_if(r.shapes.begin(), r.shapes.end(),
+                                      [&](const bst_fwd_config_t& c) { return c.chunk_pairs == most; }),
+                       r.shapes.end());
+    }
+}
+
 }  // namespace bsth
 
 // Record a timing mark on `st` after a launch of `stage` (or a start mark

@@ -250,11 +250,7 @@ int bst_plan_fft_length(bst_plan_t p) { return p ? p->M : 0; }
 
 size_t bst_workspace_bytes(bst_plan_t p, int slices) {
     if (!p || slices <= 0) return 0;
-    const int pairs = (slices + 1) / 2;
-    const int chunk = bsth::fwd_chunk(p, pairs, p->chunk_pairs);
-    const int nchunks = (pairs + chunk - 1) / chunk;
-    const int lanes = std::min(std::min(nchunks, bsth::kMaxLanes), std::max(p->max_lanes, 1));   // chunks in flight
-    return (size_t)lanes * chunk * bsth::fwd_bytes_per_pair(p) + bsth::prep_table_bytes(p);
+    return bsth::fwd_ws_bytes(p, slices, p->chunk_pairs);
 }
 
 size_t bst_adjoint_workspace_bytes(bst_plan_t p, int slices) {
@@ -376,28 +372,6 @@ bst_status_t bst_plan_get_forward_config(bst_plan_t p, bst_fwd_config_t* c) {
     return BST_OK;
 }
 
-// The candidate launch shapes of the autotuner: for bilinear plans the
-// interleaved layout (where the length has it) and the paired one; half the
-// default chunk, the default and twice it (a larger chunk fills more waves of
-// blocks, a smaller one keeps the intermediates in L2); either block order.  The
-// lane count stays the plan's.  Radix 8 (never fewer passes), the packed layout
-// and the paired gather through shared memory measured slower at every length
-// and are left to bst_plan_set_forward_config.
-static std::vector<bst_fwd_config_t> tune_candidates(const bst_plan_s* p) {
-    std::vector<bst_fwd_config_t> out;
-    std::vector<int> layouts;
-    if (p->grid_kind != BST_GRID_BILINEAR) {
-        layouts = {BST_LAYOUT_PACKED};
-    } else {
-        if (bsth::inter_pairs_of(p->M) > 1) layouts.push_back(BST_LAYOUT_INTERLEAVED);
-        layouts.push_back(BST_LAYOUT_PAIRED);
-    }
-    for (int l : layouts)
-        for (int ch : {p->chunk_default / 2, p->chunk_default, std::min(256, 2 * p->chunk_default)})
-            for (int pf : {0, 1}) out.push_back(bst_fwd_config_t{16, l, ch, pf, p->max_lanes, 1});
-    return out;
-}
-
 bst_status_t bst_plan_autotune(bst_plan_t p, int slices, int* chosen) {
     if (!p) return BST_ERR_INVALID_ARGUMENT;
     if (!bsth::on_plan_device(p)) return BST_ERR_INVALID_ARGUMENT;
@@ -405,18 +379,14 @@ bst_status_t bst_plan_autotune(bst_plan_t p, int slices, int* chosen) {
         const size_t per = (size_t)p->V * p->N * sizeof(float);
         slices = (int)std::max<size_t>(4, std::min<size_t>(4096, (((size_t)256 << 20) / per) & ~(size_t)1));
     }
-    // at least one chunk of the largest candidate on each lane
-    slices = std::max(slices, 2 * 2 * std::min(256, 2 * p->chunk_default));
+    size_t free_bytes = 0, total_bytes = 0;
+    if (cudaMemGetInfo(&free_bytes, &total_bytes) != cudaSuccess) return BST_ERR_CUDA;
     bst_fwd_config_t old{};
     bst_plan_get_forward_config(p, &old);
-    const std::vector<bst_fwd_config_t> cand = tune_candidates(p);
-    // workspace for the largest candidate chunk
-    size_t nws = 0;
-    for (const bst_fwd_config_t& c : cand) {
-        bst_plan_set_forward_config(p, &c);
-        nws = std::max(nws, bst_workspace_bytes(p, slices));
-    }
-    bst_plan_set_forward_config(p, &old);
+    const bsth::TuneRun run = bsth::tune_run(p, slices, free_bytes / 2);
+    const std::vector<bst_fwd_config_t>& cand = run.shapes;
+    const size_t nws = run.ws;
+    slices = run.slices;
     const size_t nin = (size_t)slices * p->V * p->N, nout = (size_t)slices * p->N * p->N;
     float *in = nullptr, *out = nullptr;
     void* ws = nullptr;

@@ -49,8 +49,40 @@ static void forward() {
     CHECK(plan(2048, 2048, 2, 4 * GiB).chunk_pairs == 1);
 }
 
+// What the autotuner allocates: the rays, the volume and the largest workspace.
+static void autotuner() {
+    struct { int N, V, alpha; size_t room; } cases[] = {
+        {2048, 2048, 2, 135 * GiB}, {2048, 2048, 2, 3 * GiB}, {2048, 2048, 2, GiB}, {4096, 20000, 1, 135 * GiB},
+        {4096, 20000, 1, 20 * GiB}, {4096, 20000, 1, 4 * GiB}, {512, 512, 2, 135 * GiB}, {64, 64, 2, GiB / 2},
+        {8, 8, 2, GiB}};
+    for (const auto& c : cases)
+        for (int kind : {BST_GRID_BILINEAR, BST_GRID_KAISER_BESSEL})
+            for (int slices : {4, 64, 4096})
+                for (int lanes : {1, 2}) {
+                    bst_plan_s p = plan(c.N, c.V, c.alpha, 2 * c.room);
+                    p.grid_kind = kind;
+                    p.max_lanes = lanes;
+                    const bsth::TuneRun r = bsth::tune_run(&p, slices, c.room);
+                    CHECK(!r.shapes.empty() && r.slices >= 2);
+                    size_t ws = 0;
+                    int most = 0;
+                    for (const bst_fwd_config_t& s : r.shapes) {
+                        CHECK(s.chunk_pairs >= 1 && s.chunk_pairs <= 256);
+                        most = std::max(most, s.chunk_pairs);
+                        ws = std::max(ws, bsth::fwd_ws_bytes(&p, r.slices, s.chunk_pairs));
+                    }
+                    CHECK(ws == r.ws);
+                    CHECK(r.ws + ((size_t)c.V * c.N + (size_t)c.N * c.N) * sizeof(float) * r.slices <= c.room);
+                    if (c.room > 100 * GiB && slices < 4096) {   // everything fits: all candidates, the slices asked for
+                        CHECK(most == std::min(256, 2 * p.chunk_default));
+                        CHECK(r.slices == std::max(slices, 4 * most));
+                    }
+                }
+}
+
 int main() {
     forward();
+    autotuner();
     if (!bad) std::printf("OK\n");
     return bad != 0;
 }
