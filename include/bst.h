@@ -159,7 +159,11 @@ bst_status_t bst_fbp_prep(bst_plan_t plan, const float* d_sino, int slices,
                           float kb_beta, float kb_halfwidth, const float* d_g,
                           float* d_volume, void* d_ws, size_t ws_bytes, bst_stream_t stream);
 
-/* Device workspace in bytes for radon_adjoint and bst_fbp_filter_grad. */
+/* Device workspace in bytes for radon_adjoint, bst_fbp_filter_grad and
+ * bst_fbp_backward: the slice pairs in flight, up to about 512 MiB of them and at
+ * least one group of the polar kernel (four pairs, two from M = 3072), or fewer, down
+ * to one pair, where that exceeds a sixteenth of the device memory free at the
+ * plan's creation. */
 size_t bst_adjoint_workspace_bytes(bst_plan_t plan, int slices);
 
 /* Exact adjoint (transpose) of the discrete operator of bst_fbp (mode

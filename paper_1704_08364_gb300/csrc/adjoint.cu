@@ -517,20 +517,8 @@ struct AdjLayout {
     float* part;
 };
 
-static size_t adj_rows_t(const bst_plan_s* p) { return (size_t)((p->N + 3) / 4) * 4; }
-
-static size_t adj_bytes_per_pair(const bst_plan_s* p) {
-    return (std::max(adj_rows_t(p), (size_t)p->V) * p->M + (size_t)p->M * p->M) * sizeof(float2);
-}
-
-// Pairs in flight: as many as fit in 512 MiB, whole groups of four where there
-// are more, and at least the pairs that the polar kernel takes together.
-static int adj_chunk(const bst_plan_s* p, int pairs) {
-    const size_t budget = (size_t)512 << 20;
-    size_t c = std::max<size_t>(p->M >= 3072 ? 2 : 4, budget / adj_bytes_per_pair(p));
-    if (c > 4) c &= ~(size_t)3;
-    return (int)std::min<size_t>((size_t)pairs, c);
-}
+using bsth::adj_chunk;
+using bsth::adj_rows_t;
 
 // pairs that X holds: a rest of three is a group of four
 static size_t adj_x_pairs(const bst_plan_s* p, int chunk) {

@@ -46,7 +46,7 @@ struct bst_plan_s {
     int kb_nstrips = 0;
     int chunk_pairs = 1;            // slice pairs per chunk of the forward path
     int chunk_default = 1;          // the chunk that the plan started with (bsth::default_chunk)
-    size_t ws_most = 0;             // bytes of a workspace that more than one pair a lane may take
+    size_t ws_most = 0;             // bytes of a workspace with more than one pair in flight
     int maxr = 16;                  // FFT radix schedule of the forward path (16 or 8; autotuned)
     int fwd_layout = 0;             // BST_LAYOUT_PACKED or BST_LAYOUT_PAIRED (autotuned)
     int pair_fast = 0;              // gridding blocks ordered pair-fastest (autotuned)
@@ -146,8 +146,8 @@ __host__ __device__ constexpr int inter_pairs_of(int M) {
     return c > 0 && tpl % (16 / c) == 0 ? c : 1;
 }
 
-// Bytes that the forward workspace of a plan may take with more than one slice pair a
-// lane: 4 GiB, less where little device memory is free at the plan's creation.
+// Bytes that a workspace of a plan may take with more than one slice pair in flight (a
+// lane, on the forward path): 4 GiB, less where little device memory is free at the plan's creation.
 inline size_t workspace_most(size_t free_bytes) { return std::min<size_t>((size_t)4 << 30, free_bytes / 16); }
 
 // Slice pairs per chunk that a plan starts with: 64 MiB of workspace, but at least 8
@@ -188,6 +188,23 @@ inline size_t fwd_ws_bytes(const bst_plan_s* p, int slices, int most) {
     const int nchunks = (pairs + chunk - 1) / chunk;
     const int lanes = std::min(std::min(nchunks, kMaxLanes), std::max(p->max_lanes, 1));   // chunks in flight
     return (size_t)lanes * chunk * fwd_bytes_per_pair(p) + prep_table_bytes(p);
+}
+
+// rows of T of a slice pair; bytes of a slice pair of the adjoint and the filter gradient
+inline size_t adj_rows_t(const bst_plan_s* p) { return (size_t)((p->N + 3) / 4) * 4; }
+inline size_t adj_bytes_per_pair(const bst_plan_s* p) {
+    return (std::max(adj_rows_t(p), (size_t)p->V) * p->M + (size_t)p->M * p->M) * sizeof(float2);
+}
+
+// Slice pairs that the adjoint has in flight: as many as fit in 512 MiB, whole groups
+// of four where there are more, and at least the pairs that the polar kernel takes
+// together; fewer, down to one, where that exceeds the plan's bound.
+inline int adj_chunk(const bst_plan_s* p, int pairs) {
+    const size_t per = adj_bytes_per_pair(p), group = p->M >= 3072 ? 2 : 4;
+    size_t c = std::max(std::min(group, p->ws_most / per), std::min<size_t>((size_t)512 << 20, p->ws_most) / per);
+    if (c > 4) c &= ~(size_t)3;
+    else if (c == 3 && group == 4) c = 2;   // three take the space of four
+    return (int)std::min<size_t>((size_t)pairs, std::max<size_t>(c, 1));
 }
 
 // The candidate launch shapes of the autotuner, largest chunk first: for bilinear

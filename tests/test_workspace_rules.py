@@ -15,7 +15,8 @@ NVCC = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "bin", "nvcc
 
 
 def test_workspace_sizes_are_bounded(tmp_path):
-    """tests/workspace_check.cu: the chunk that a plan starts with, what the autotuner allocates."""
+    """tests/workspace_check.cu: the chunk that a plan starts with, what the autotuner
+    allocates, and the pairs that the adjoint has in flight."""
     nvcc = NVCC if os.path.exists(NVCC) else shutil.which("nvcc")
     if not nvcc:
         pytest.skip("nvcc not available")

@@ -80,8 +80,26 @@ static void autotuner() {
                 }
 }
 
+// The adjoint: a pair alone, or what stays within the bound.
+static void adjoint() {
+    const int N[] = {8, 48, 512, 1024, 1536, 2048}, V[] = {2, 64, 2048, 20000};
+    const size_t free_bytes[] = {GiB / 4, GiB, 4 * GiB, 270 * GiB};
+    for (int n : N)
+        for (int v : V)
+            for (size_t f : free_bytes)
+                for (int pairs : {1, 2, 3, 5, 64, 1000}) {
+                    const bst_plan_s p = plan(n, v, 2, f);
+                    const int c = bsth::adj_chunk(&p, pairs);
+                    CHECK(c >= 1 && c <= pairs);
+                    CHECK(c == 1 || c * bsth::adj_bytes_per_pair(&p) <= f / 16);
+                }
+    const bst_plan_s p = plan(1024, 1024, 2, 270 * GiB), q = plan(2048, 2048, 2, 270 * GiB);
+    CHECK(bsth::adj_chunk(&p, 64) == 8 && bsth::adj_chunk(&p, 3) == 3 && bsth::adj_chunk(&q, 64) == 2);
+}
+
 int main() {
     forward();
+    adjoint();
     autotuner();
     if (!bad) std::printf("OK\n");
     return bad != 0;
