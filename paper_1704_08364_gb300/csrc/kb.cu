@@ -15,11 +15,10 @@
 #include <cmath>
 #include <cstdint>
 #include <new>
-#include <system_error>
-#include <thread>
 #include <vector>
 
 #include "bst_kb.cuh"
+#include "bst_parallel.h"
 
 namespace bst {
 
@@ -129,27 +128,6 @@ static bool upload_vec(T** d, const std::vector<T>& h) {
     return h.empty() || cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
-// fn(begin, end) over [0, n) in up to 8 host threads; on the calling thread alone
-// where a thread cannot be started.  fn must not throw (it allocates nothing).
-template <class F>
-static void parallel(int n, F&& fn) {
-    const int most = std::min({8, n, (int)std::max(1u, std::thread::hardware_concurrency())});
-    std::vector<std::thread> t;
-    t.reserve(most);
-    int at = 0;
-    for (int i = 0; i + 1 < most; ++i) {
-        const int end = (int)((long long)n * (i + 1) / most);
-        try {
-            t.emplace_back([&fn, at, end] { fn(at, end); });
-        } catch (const std::system_error&) {
-            break;
-        }
-        at = end;
-    }
-    fn(at, n);
-    for (std::thread& x : t) x.join();
-}
-
 // Tables of KB gridding of width W for the plan, host-built in double:
 //   the kernel polynomial and the deapodization;
 //   per strip of two columns, every sample (j, k), k != 0, -M/2, whose
@@ -227,7 +205,7 @@ static bst_status_t build_kb(bst_plan_s* p, int W) {
         const int f = (int)std::floor(x - 0.5 * W) + 1;
         return (uint16_t)(f < 0 ? f + M : (f >= M ? f - M : f));
     };
-    parallel(V, [&](int j0, int j1) {
+    bsth::parallel(V, [&](int j0, int j1) {
         for (int j = j0; j < j1; ++j) {
             const double c = std::cos(p->theta[j]), s = std::sin(p->theta[j]);
             for (int i = 0; i < M; ++i) {
@@ -254,7 +232,7 @@ static bst_status_t build_kb(bst_plan_s* p, int W) {
     const int wrap = std::min(bst::KB_WMAX, M);
     std::vector<int> row((size_t)ns * (M + 1), 0);   // row[s][r]: entries of the strip with first row < r
     std::vector<size_t> start(ns + 1, 0);            // the strip's place in the list
-    parallel(ns, [&](int s0, int s1) {
+    bsth::parallel(ns, [&](int s0, int s1) {
         each(s0, s1, [&](int s, int r, int) { ++row[(size_t)s * (M + 1) + r + 1]; });
         for (int s = s0; s < s1; ++s)
             for (int r = 0; r < M; ++r) row[(size_t)s * (M + 1) + r + 1] += row[(size_t)s * (M + 1) + r];
@@ -289,7 +267,7 @@ static bst_status_t build_kb(bst_plan_s* p, int W) {
     }
     std::vector<int> list(n), fill((size_t)ns * M);
     std::vector<int4> items(istart[ns]);
-    parallel(ns, [&](int s0, int s1) {
+    bsth::parallel(ns, [&](int s0, int s1) {
         for (int s = s0; s < s1; ++s)
             for (int r = 0; r < M; ++r) fill[(size_t)s * M + r] = pos(s, r);
         each(s0, s1, [&](int s, int r, int at) { list[fill[(size_t)s * M + r]++] = at; });
