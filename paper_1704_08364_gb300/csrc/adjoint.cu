@@ -518,18 +518,12 @@ struct AdjLayout {
 };
 
 using bsth::adj_chunk;
+using bsth::adj_fg_blocks;
 using bsth::adj_rows_t;
 
 // pairs that X holds: a rest of three is a group of four
 static size_t adj_x_pairs(const bst_plan_s* p, int chunk) {
     return (size_t)chunk + (p->M < 3072 && chunk % 4 == 3 ? 1 : 0);
-}
-
-// two blocks an SM over the chunk's pairs
-static int adj_fg_blocks(const bst_plan_s* p, int chunk) {
-    const int tpl = (p->M % 3 == 0) ? p->M / 12 : p->M / 16;
-    const int lpc = std::max(1, 256 / tpl);
-    return std::max(1, std::min((p->V + lpc - 1) / lpc, (304 + chunk - 1) / chunk));
 }
 
 static AdjLayout adj_layout(const bst_plan_s* p, int pairs, void* ws) {

@@ -349,22 +349,11 @@ bst_status_t bst_launch_brute(bst_plan_s* p, const float* sino, int slices, cons
         if (s != BST_OK) return s;
         y = q;
     }
-    // Slices and pixels a thread, by the blocks per SM that each shape gives.  Eight
-    // slices (four pixels) read a window for twice the slices, but a block takes
-    // 7/4 of the time of one of four slices, and below three blocks an SM its longer
-    // chain shows.  With four slices, more pixels a thread do less work in all, and
-    // fewer have the shorter chain.  300 angles, us with one, two, four pixels: 64 x 64
-    // 57, 61, 77; 16 slices of 192 x 192 130, 89, 91; 5 of 384 x 384 228, 165, 126;
-    // four and eight slices: 20 of 512 x 512 467, 494; 40 904, 754.
-    const auto blocks = [&](int h, int r) {
-        return (long long)((p->N + 31) / 32) * ((p->N + 4 * r - 1) / (4 * r)) * ((slices + 4 * h - 1) / (4 * h));
-    };
-    constexpr long long SMS = 152;
-    const long long b4 = blocks(1, 4), c4 = (b4 + SMS - 1) / SMS, c8 = (blocks(2, 4) + SMS - 1) / SMS;
+    const bsth::SsShape sh = bsth::ss_shape(p->N, slices, p->sms);
     bst_timing_mark(p, st, -1);
-    if (c8 >= 3 && 7 * c8 < 4 * c4) bst::launch_ss_bp<2, 4>(p, y, slices, vol, st);
-    else if (5 * b4 > 12 * SMS) bst::launch_ss_bp<1, 4>(p, y, slices, vol, st);
-    else if (blocks(1, 1) > SMS) bst::launch_ss_bp<1, 2>(p, y, slices, vol, st);
+    if (sh.h == 2) bst::launch_ss_bp<2, 4>(p, y, slices, vol, st);
+    else if (sh.r == 4) bst::launch_ss_bp<1, 4>(p, y, slices, vol, st);
+    else if (sh.r == 2) bst::launch_ss_bp<1, 2>(p, y, slices, vol, st);
     else bst::launch_ss_bp<1, 1>(p, y, slices, vol, st);
     bst_timing_mark(p, st, 4);
     return cudaGetLastError() == cudaSuccess ? BST_OK : BST_ERR_CUDA;

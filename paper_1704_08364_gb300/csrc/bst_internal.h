@@ -13,6 +13,7 @@
 struct bst_plan_s {
     int N = 0, V = 0, M = 0, alpha = 0;
     int device = 0;
+    int sms = 0;                    // multiprocessors of the device
     std::vector<double> theta;      // angles as given (float32 widened exactly)
     // device tables owned by the plan
     float2* tw = nullptr;           // [M] exp(-2 pi i m / M)
@@ -205,6 +206,33 @@ inline int adj_chunk(const bst_plan_s* p, int pairs) {
     if (c > 4) c &= ~(size_t)3;
     else if (c == 3 && group == 4) c = 2;   // three take the space of four
     return (int)std::min<size_t>((size_t)pairs, std::max<size_t>(c, 1));
+}
+
+// Angle blocks per pair of the filter gradient: two blocks an SM over the chunk's pairs.
+inline int adj_fg_blocks(const bst_plan_s* p, int chunk) {
+    const int tpl = (p->M % 3 == 0) ? p->M / 12 : p->M / 16;
+    const int lpc = std::max(1, 256 / tpl);
+    return std::max(1, std::min((p->V + lpc - 1) / lpc, (2 * p->sms + chunk - 1) / chunk));
+}
+
+// Slant stack: 4 h slices and r pixels a thread, by the blocks per SM that each shape
+// gives.  Eight slices (four pixels) read a window for twice the slices, but a block
+// takes 7/4 of the time of one of four slices, and below three blocks an SM its longer
+// chain shows.  With four slices, more pixels a thread do less work in all, and
+// fewer have the shorter chain.  300 angles, us with one, two, four pixels: 64 x 64
+// 57, 61, 77; 16 slices of 192 x 192 130, 89, 91; 5 of 384 x 384 228, 165, 126;
+// four and eight slices: 20 of 512 x 512 467, 494; 40 904, 754.
+struct SsShape {
+    int h, r;
+};
+inline SsShape ss_shape(int N, int slices, int sms) {
+    const auto blocks = [&](int h, int r) {
+        return (long long)((N + 31) / 32) * ((N + 4 * r - 1) / (4 * r)) * ((slices + 4 * h - 1) / (4 * h));
+    };
+    const long long b4 = blocks(1, 4), c4 = (b4 + sms - 1) / sms, c8 = (blocks(2, 4) + sms - 1) / sms;
+    if (c8 >= 3 && 7 * c8 < 4 * c4) return {2, 4};
+    if (5 * b4 > 12 * sms) return {1, 4};
+    return {1, blocks(1, 1) > sms ? 2 : 1};
 }
 
 // The candidate launch shapes of the autotuner, largest chunk first: for bilinear

@@ -156,7 +156,12 @@ bst_status_t bst_plan_create(bst_plan_t* out, int rays, int angles, const float*
     p->M = M;
     p->alpha = pad_factor;
     p->theta = th;
-    cudaGetDevice(&p->device);
+    if (cudaGetDevice(&p->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
+        cudaGetLastError();
+        free_plan(p);
+        return BST_ERR_CUDA;
+    }
     const int V = angles;
 
     // twiddles: the base table, then each radix schedule's per-pass tables

@@ -1,5 +1,6 @@
 // Test-only host program (compiled and run by tests/test_workspace_rules.py, no
-// GPU needed): how many slice pairs the workspaces of a plan are sized for.
+// GPU needed): how many slice pairs the workspaces of a plan are sized for, and the
+// rules that ask for the device's number of SMs.
 #include <cstdio>
 
 #include "bst_internal.h"
@@ -97,7 +98,23 @@ static void adjoint() {
     CHECK(bsth::adj_chunk(&p, 64) == 8 && bsth::adj_chunk(&p, 3) == 3 && bsth::adj_chunk(&q, 64) == 2);
 }
 
+// Shapes by the blocks per SM: the same number of blocks an SM gives the same shape.
+static void per_sm() {
+    auto is = [](bsth::SsShape s, int h, int r) { return s.h == h && s.r == r; };
+    CHECK(is(bsth::ss_shape(512, 16, 152), 2, 4) && is(bsth::ss_shape(512, 20, 152), 1, 4));
+    CHECK(is(bsth::ss_shape(512, 8, 152), 1, 4) && is(bsth::ss_shape(192, 16, 152), 1, 2));
+    CHECK(is(bsth::ss_shape(64, 1, 152), 1, 1) && is(bsth::ss_shape(64, 1, 16), 1, 2));
+    CHECK(is(bsth::ss_shape(512, 16, 8), 2, 4) && is(bsth::ss_shape(192, 16, 19), 2, 4));
+    CHECK(is(bsth::ss_shape(512, 16, 1520), 1, 2) && is(bsth::ss_shape(192, 16, 1520), 1, 1));
+    bst_plan_s p = plan(1024, 1024, 2, 270 * GiB);
+    for (int sms : {8, 148, 152}) {
+        p.sms = sms;
+        CHECK(bsth::adj_fg_blocks(&p, 8) == (2 * sms + 7) / 8 && bsth::adj_fg_blocks(&p, 1000) == 1);
+    }
+}
+
 int main() {
+    per_sm();
     forward();
     adjoint();
     autotuner();
