@@ -594,8 +594,10 @@ static bst_status_t adjoint_chunk(bst_plan_s* p, const AdjLayout& L, const float
     for (int stage = 0; stage < 2; ++stage) {
         if (full > 0) adjoint_group<M, PM>(p, L, stage, slices, p0, 0, full, mode, g, sino, keep_lam, st);
         if (rem == 1) adjoint_group<M, 1>(p, L, stage, slices, p0, full, 1, mode, g, sino, keep_lam, st);
-        if (rem == 2) adjoint_group<M, 2>(p, L, stage, slices, p0, full, 2, mode, g, sino, keep_lam, st);
-        if (rem == 3) adjoint_group<M, PM>(p, L, stage, slices, p0, full, 3, mode, g, sino, keep_lam, st);
+        if constexpr (PM > 2) {
+            if (rem == 2) adjoint_group<M, 2>(p, L, stage, slices, p0, full, 2, mode, g, sino, keep_lam, st);
+            if (rem == 3) adjoint_group<M, PM>(p, L, stage, slices, p0, full, 3, mode, g, sino, keep_lam, st);
+        }
     }
     return BST_OK;
 }

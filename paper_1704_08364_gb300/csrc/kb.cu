@@ -77,7 +77,9 @@ bst_status_t launch_kb_col_M(bst_plan_s* p, const float2* Z, float2* T, int np, 
     bst_status_t s = BST_OK;
     if (full > 0) s = launch_kb_col_P<M, MAXR, PM>(p, a, Z, T, full, st);
     if (s == BST_OK && rem == 1) s = launch_kb_col_P<M, MAXR, 1>(p, a, Z + full * zs, T + full * ts, 1, st);
-    if (s == BST_OK && rem == 2) s = launch_kb_col_P<M, MAXR, 2>(p, a, Z + full * zs, T + full * ts, 2, st);
+    if constexpr (PM > 2) {
+        if (s == BST_OK && rem == 2) s = launch_kb_col_P<M, MAXR, 2>(p, a, Z + full * zs, T + full * ts, 2, st);
+    }
     return s;
 }
 
