@@ -39,7 +39,7 @@ template <int M> __host__ __device__ constexpr int inter_stride(int n) { return 
 // Place of slot k, sign s (0: +k, 1: -k) in a row, in complex values: [k][s][P],
 // for P = 2 [k / 2][s][k % 2][P], so that the ray kernel writes whole sectors there
 // too (consecutive bins of one sign).
-template <int P> __device__ __forceinline__ int inter_slot(int k, int s) {
+template <int P> __host__ __device__ __forceinline__ int inter_slot(int k, int s) {
     return P == 2 ? (k >> 1) * 8 + s * 4 + (k & 1) * 2 : (k * 2 + s) * P;
 }
 
