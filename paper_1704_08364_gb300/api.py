@@ -94,18 +94,19 @@ class Plan:
             self._ws[key] = buf
         return buf
 
-    def _chunked_workspace(self, kind: str, size, slices: int, device) -> torch.Tensor:
-        """The workspace of a chunked forward call, size(handle, slices) bytes.  Where
-        it cannot be allocated the plan goes on with chunks of half as many pairs,
+    def _smaller_workspace(self, kind: str, size, slices: int, device) -> torch.Tensor:
+        """The workspace of a chunked forward call, size(handle, slices) bytes, after it
+        could not be allocated: the plan goes on with chunks of half as many pairs,
         down to one pair, the least that the path takes."""
         while True:
+            pairs = min(self.forward_config["chunk_pairs"], (slices + 1) // 2)
+            if pairs <= 1:
+                return self.workspace(kind, size(self._h, slices), device)
+            self.set_forward_config(chunk_pairs=pairs // 2)
             try:
                 return self.workspace(kind, size(self._h, slices), device)
             except torch.OutOfMemoryError:
-                pairs = min(self.forward_config["chunk_pairs"], (slices + 1) // 2)
-                if pairs <= 1:
-                    raise
-                self.set_forward_config(chunk_pairs=pairs // 2)
+                pass
 
     def workspace_bytes(self, slices: int) -> int:
         return int(self._lib.bst_workspace_bytes(self._h, int(slices)))
@@ -221,7 +222,10 @@ class Plan:
         if g is not None:
             _need(g, "g", (self.M // 2,))
         out = self._volume(out, S, sino)
-        ws = self._chunked_workspace("fwd", self._lib.bst_workspace_bytes, S, sino.device)
+        try:
+            ws = self.workspace("fwd", self._lib.bst_workspace_bytes(self._h, S), sino.device)
+        except torch.OutOfMemoryError:
+            ws = self._smaller_workspace("fwd", self._lib.bst_workspace_bytes, S, sino.device)
         if mode == FILTER:
             code = self._lib.bst_fbp(self._h, _ptr(sino), S, _ptr(g), _ptr(out), _ptr(ws), ws.numel(), _stream())
             _check(code, "bst_fbp")
@@ -250,7 +254,10 @@ class Plan:
         if out is None:
             out = torch.empty((S, self.rays, self.rays), dtype=torch.float32, device=sino.device)
         _need(out, "out", (S, self.rays, self.rays))
-        ws = self._chunked_workspace("fwd", self._lib.bst_workspace_bytes, S, sino.device)
+        try:
+            ws = self.workspace("fwd", self._lib.bst_workspace_bytes(self._h, S), sino.device)
+        except torch.OutOfMemoryError:
+            ws = self._smaller_workspace("fwd", self._lib.bst_workspace_bytes, S, sino.device)
         _check(self._lib.bst_fbp_prep(self._h, _ptr(sino), S, _ptr(dark), _ptr(flat), float(shift), float(kb_beta),
                                       float(kb_halfwidth), _ptr(g), _ptr(out), _ptr(ws), ws.numel(), _stream()),
                "bst_fbp_prep")
@@ -290,7 +297,10 @@ class Plan:
         if g is not None:
             _need(g, "g", (self.M // 2,))
         dev = device or torch.device("cuda", torch.cuda.current_device())
-        ws = self._chunked_workspace("host", self._lib.bst_host_workspace_bytes, S, dev)
+        try:
+            ws = self.workspace("host", self._lib.bst_host_workspace_bytes(self._h, S), dev)
+        except torch.OutOfMemoryError:
+            ws = self._smaller_workspace("host", self._lib.bst_host_workspace_bytes, S, dev)
         _check(self._lib.bst_fbp_host(self._h, _ptr(sino), S, _ptr(g), _ptr(out), _ptr(ws), ws.numel(), _stream()),
                "bst_fbp_host")
         torch.cuda.current_stream().synchronize()
