@@ -95,7 +95,18 @@ def stage_flops(N: int, V: int, M: int, kb_width: int = 0) -> dict:
 
 STAGE_NAMES = {0: "k_ray_fft", 1: "k_grid_col", 2: "k_row_ifft", 3: "k_ss_filter", 4: "k_ss_bp"}
 
-# DRAM bytes (read + write) per launch of each forward kernel from one ncu
+
+def kernel_names(config: dict, kb: bool) -> dict:
+    """The forward kernels that a launch shape runs on whole groups of slice pairs."""
+    if kb:
+        return {0: "k_ray_fft", 1: "k_kb_col", 2: "k_row_ifft"}
+    if config["layout"] == "interleaved":
+        return {0: "k_ray_inter", 1: "k_grid_inter", 2: "k_row_inter"}
+    grid = {"packed": "k_grid_col", "paired": "k_grid_col_xchg" if config["grid_xchg"] else "k_grid_col_paired"}
+    return {0: "k_ray_fft", 1: grid[config["layout"]], 2: "k_row_ifft"}
+
+
+# DRAM bytes (read + write) per launch of each forward stage (keyed by STAGE_NAMES) from one ncu
 # capture of the dram__bytes_read.sum and dram__bytes_write.sum counters on
 # the volume-2048 geometry (64 slices: launches of 16 pairs each, cold cache), keyed by
 # a SHA-256 over the kernels' device-code headers (the host launcher lives in
@@ -571,9 +582,7 @@ def run_ours(args, rank, world):
     stage_ms = {s: sms[s] for s in range(3)}
     stage_n = {s: sl[s] for s in range(3)}
     flops = stage_flops(N, V, M, kbw)
-    names = dict(STAGE_NAMES)
-    if kbw:
-        names[1] = "k_kb_col"
+    names = kernel_names(tuned, bool(kbw))
     dom = max(stage_ms, key=lambda s: stage_ms[s])
     # slice pairs per launch: the tuned chunk (the last chunk of a step may be
     # shorter; the average below counts launches, so use whole-step pairs)
@@ -583,7 +592,7 @@ def run_ours(args, rank, world):
     peak_tf = fp32_peak_tflops(sm_max)
     flops = {k: v * pairs_per_launch for k, v in flops.items()}
     achieved_tf = flops[dom] / (avg_ms / 1e3) / 1e12
-    traffic = None if kbw else captured_traffic(names[dom], N, alpha, tuned)
+    traffic = None if kbw else captured_traffic(STAGE_NAMES[dom], N, alpha, tuned)
     # the bound is whichever floor is higher for this kernel: its algorithmic
     # flops at the FP32 peak, or its compulsory bytes (its own inputs and
     # outputs read or written once) at the HBM peak
