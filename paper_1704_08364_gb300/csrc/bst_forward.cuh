@@ -29,8 +29,8 @@
 //               rows at a time, keep the N central columns, scale by
 //               dt dw^2 = N / (2 M^2), write Re to slice a and Im to slice b.
 //
-// Z and T live in a caller-provided workspace sized for a chunk of pairs
-// that fits in L2 where possible (one pair at N = 2048: 2 x 64 MiB).
+// Z and T live in a caller-provided workspace sized for a chunk of pairs (128 MiB
+// a pair at N = V = 2048, pad factor 2).
 // This header holds device code only; the host launcher is bst_launch.cuh.
 #pragma once
 #include <cuda_runtime.h>

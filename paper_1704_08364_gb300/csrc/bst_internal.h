@@ -48,11 +48,11 @@ struct bst_plan_s {
     int chunk_pairs = 1;            // slice pairs per chunk of the forward path
     int chunk_default = 1;          // the chunk that the plan started with (bsth::default_chunk)
     size_t ws_most = 0;             // bytes of a workspace with more than one pair in flight
-    int maxr = 16;                  // FFT radix schedule of the forward path (16 or 8; autotuned)
-    int fwd_layout = 0;             // BST_LAYOUT_PACKED or BST_LAYOUT_PAIRED (autotuned)
+    int maxr = 16;                  // FFT radix schedule of the forward path (16 or 8)
+    int fwd_layout = 0;             // a bst_layout_t (interleaved at creation; autotuned)
     int pair_fast = 0;              // gridding blocks ordered pair-fastest (autotuned)
     int max_lanes = 2;              // streams alternating chunks (1 or 2)
-    int grid_xchg = 0;              // register-fed paired gridding (0 or 1; autotuned)
+    int grid_xchg = 0;              // register-fed paired gridding (0 or 1)
     // two plan-owned streams that alternate chunks of the forward path (fork
     // from and join back to the caller's stream with events), created on first use
     cudaStream_t lane[3] = {nullptr, nullptr, nullptr};

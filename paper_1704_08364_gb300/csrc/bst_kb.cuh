@@ -22,9 +22,8 @@
 // band's 2 x 4 cell of every pair in registers (the weight of every sample at
 // every cell point, zero outside the footprint), add the four partial cells by
 // shuffles and store the sum (or add it atomically, if the band has several
-// items: those near the origin, where the samples crowd); the list is read 16
-// bytes at a time.  A warp takes eight items at once, longest first, from a
-// shared counter.  Then the inverse FFT along r' of each column runs in place
+// items: those near the origin, where the samples crowd).  A warp takes eight items
+// at once, longest first, from a shared counter.  Then the inverse FFT along r' of each column runs in place
 // and the N central rows go to T exactly as with the bilinear gather.  The V
 // samples of the DC bin all sit at the origin; one warp sums them (with their
 // angular weights) and spreads the sum once.
