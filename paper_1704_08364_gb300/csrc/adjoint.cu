@@ -267,8 +267,9 @@ struct SinoCrop {
 // once per sample and pair instead (four times, 8 bytes of each 32-byte sector)
 // waited on the list-to-point chains (16 stall cycles per issue): 486 us for
 // the 8 pairs of 16 x 1024 x 1024, 280 us with this form and 221 us with the next
-// cell's list bounds read ahead.  What bounds it
-// now is the latency and sector traffic of the point reads from L2.
+// cell's list bounds read ahead.  What bounds it now is the latency of the chain
+// from a list entry to its point (two thirds of the stall cycles), with the L1
+// wavefronts of the point reads at 65 to 68 % of the peak.
 template <int M, int TPL, int LINES, int P, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT)
     k_adj_polar(const float2* __restrict__ X, Cells cl, int V, int N, int slices, int pair0, int npairs, int mode,

@@ -124,13 +124,13 @@ __device__ __forceinline__ void fma_slices(float2 (&acc)[H][2], float w, const f
 // shared-memory wavefronts on average with R = 4 against 16 for two reads per
 // pixel and slice.  A batch of angles with a value that is not finite reads the
 // two samples of each pixel instead (a zero weight would not hide it).  What
-// bounds it: FP32 issue and the shared-memory wavefronts, about alike, and with
-// few blocks the chain of a batch: staging loads, barrier, sums.  The loads of a
+// bounds it: FP32 issue (64 to 70 %) and the shared-memory wavefronts (61 to 71 %),
+// about alike, and with few blocks the chain of a batch: staging loads, barrier, sums.  The loads of a
 // warp for a whole batch are issued together, and the next batch's geometry with
 // them (six blocks of eight slices an SM leave the registers): 512 x 512, 512 angles, 16
-// slices 632 -> 555 us, 64 x 64, 300 angles, one slice 75 -> 57 us.  The form with
+// slices 632 -> 555 us (this kernel alone), 64 x 64, 300 angles, one slice 75 -> 57 us.  The form with
 // one pixel a thread, two 4-byte loads a slice and 103 warp instructions per 32
-// pixels, angle and 8 slices took 1033 us.
+// pixels, angle and 8 slices took 1033 us for the former.
 template <int H, int R>
 __global__ void __launch_bounds__(32 * SS_WARPS, H > 1 ? 6 : R > 1 ? 7 : 8)
     k_ss_bp(const float* __restrict__ y, int S, int V, int N, const double2* __restrict__ cs64,

@@ -23,9 +23,10 @@
 namespace bst {
 
 // P slice pairs per block (blockIdx.y: group of P of the np pairs).
-// What bounds it: instruction issue (about 210 instructions a sample, item and
-// four pairs, half of them the six kernel values) and the latency of the
-// samples' loads at 16 warps an SM.  With one pair a block, strips of four columns
+// What bounds it: the latency of the samples' loads at 16 warps an SM (long scoreboard
+// leads the stalls) and the L1 wavefronts of these scattered 8-byte reads (66 % of
+// the peak with four pairs a block, 59 % with two), before instruction issue (48 and
+// 57 %).  With one pair a block, strips of four columns
 // and an item a thread, every pair evaluated its own kernel values: 187 us a pair
 // at 1024 x 1024 (W = 6), 66 us with four pairs a block.
 template <int M, int MAXR, int P>
