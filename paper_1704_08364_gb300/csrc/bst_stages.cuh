@@ -19,6 +19,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "bst_fft.cuh"
 #include "bst_geo.cuh"
 #include "bst_internal.h"
@@ -503,6 +505,43 @@ template <int M> __host__ __device__ constexpr int paired_cpc() {
     return (128 / tpl_of<M>()) > 1 ? 128 / tpl_of<M>() : 1;
 }
 
+// slice pairs of a group of the interleaved layout for length M (1: none)
+template <int M> __host__ __device__ constexpr int group_pairs() { return bsth::inter_pairs_of(M); }
+
+// The sum over the angles of a pair's DC bin in one order, whichever kernel adds it, so
+// that a slice's volume does not depend on how many slices the call has: that of the
+// interleaved kernel, where thread a of the 2 TPL of a column pair adds angles a, a +
+// 2 TPL, .., W = 32 / P consecutive threads (a warp holds them for all P pairs)
+// add up by a butterfly, and their sums are added in turn.
+template <int M, int TPL> struct OriginSum {
+    static constexpr int W = 32 / group_pairs<M>();
+    template <class F> __device__ __forceinline__ static float2 strided(const F& dc, int a, int V) {
+        float2 s = make_float2(0.f, 0.f);
+#pragma unroll 2
+        for (int j = a; j < V; j += 2 * TPL) s = cadd(s, dc(j));
+        return s;
+    }
+    // sums of each W lanes of a warp, in all of them
+    __device__ __forceinline__ static float2 warp(float2 s) {
+#pragma unroll
+        for (int o = W / 2; o > 0; o >>= 1)
+            s = cadd(s, make_float2(__shfl_xor_sync(0xffffffffu, s.x, o), __shfl_xor_sync(0xffffffffu, s.y, o)));
+        return s;
+    }
+    // the whole sum by one warp, which stands in for all of the 2 TPL threads (whole warps)
+    template <class F> __device__ __forceinline__ static float2 by_warp(const F& dc, int lane, int V) {
+        float2 s = make_float2(0.f, 0.f);
+        for (int m = 0; m < 2 * TPL; m += 32) {
+            const float2 part = warp(strided(dc, lane + m, V));
+#pragma unroll
+            for (int i = 0; i < 32 / W; ++i)
+                s = cadd(s, make_float2(__shfl_sync(0xffffffffu, part.x, i * W),
+                                        __shfl_sync(0xffffffffu, part.y, i * W)));
+        }
+        return s;
+    }
+};
+
 // P0 + P5 + column P6 for CPC column pairs (q, -q), q = q0 + g, from the
 // paired spectrum layout Z2[V][M/2] (float4 slot (Z[j][k], Z[j][-k]), see
 // spec_store).  A Cartesian point (q, r') and its mirror (-q, -r') share the
@@ -625,34 +664,32 @@ __device__ __forceinline__ void grid_unit_paired(float2* smem, int q0, int V, in
         }
     }
     // the origin is single-valued: mean over angles of the DC bin (the gather
-    // stored 0 there, from thread 0 of the group, which also writes the mean).
-    // A group of 32 or more threads starts on a warp boundary (NT is then a
-    // multiple of 32), so its first warp reduces with a full-warp shuffle;
-    // smaller groups share a warp with other groups and sum serially.
+    // stored 0 there, from thread 0 of the group, which also writes the mean), in
+    // the order of OriginSum.  A group of 32 or more threads starts on a warp
+    // boundary (NT is then a multiple of 32): its first warp stands in for all of
+    // them; smaller groups share a warp with other groups and add with one thread.
+    using O = OriginSum<M, TPL>;
+    const auto dc = [&](int j) {
+        const float4 zz = __ldg(Z2 + paired_slot(j, 0, H, V));
+        return make_float2(zz.x, zz.y);
+    };
     if constexpr (NT >= 32) {
         if (live && q == 0 && lt < 32) {
-            float sx = 0.f, sy = 0.f;
-            for (int j = lt; j < V; j += 32) {
-                const float4 zz = __ldg(Z2 + paired_slot(j, 0, H, V));
-                sx += zz.x;
-                sy += zz.y;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                sx += __shfl_xor_sync(0xffffffffu, sx, o);
-                sy += __shfl_xor_sync(0xffffffffu, sy, o);
-            }
-            if (lt == 0) l0.store(0, make_float2(sx / (float)V, sy / (float)V));
+            const float2 s = O::by_warp(dc, lt, V);
+            if (lt == 0) l0.store(0, make_float2(s.x / (float)V, s.y / (float)V));
         }
     } else {
         if (live && q == 0 && lt == 0) {
-            float sx = 0.f, sy = 0.f;
-            for (int j = 0; j < V; ++j) {
-                const float4 zz = __ldg(Z2 + paired_slot(j, 0, H, V));
-                sx += zz.x;
-                sy += zz.y;
+            float2 s = make_float2(0.f, 0.f);
+            if constexpr (O::W == 4 && NT % 4 == 0) {
+                for (int a = 0; a < NT; a += 4)
+                    s = cadd(s, cadd(cadd(O::strided(dc, a, V), O::strided(dc, a + 2, V)),
+                                     cadd(O::strided(dc, a + 1, V), O::strided(dc, a + 3, V))));
+            } else {
+                static_assert(group_pairs<M>() == 1, "groups of eight pairs, or a length that has no groups");
+                for (int j = 0; j < V; ++j) s = cadd(s, dc(j));
             }
-            l0.store(0, make_float2(sx / (float)V, sy / (float)V));
+            l0.store(0, make_float2(s.x / (float)V, s.y / (float)V));
         }
     }
     sync();
@@ -676,7 +713,8 @@ __device__ __forceinline__ void grid_unit_paired(float2* smem, int q0, int V, in
 // The taps of a quarter-warp (the unit in which 16-byte loads are served)
 // are those of 8 consecutive rows of one column, as in grid_unit_paired.
 // PS point pairs per gather step.  tid: the thread among the column pair's 2 TPL
-// (whole warps; -1: threadIdx.x); `sync` the barrier that covers them.
+// (whole warps; -1: threadIdx.x); `sync` the barrier that covers them (with BlockSync
+// a block is one column pair).
 template <int M, int TPL, int MAXR, int NC = 0, int PS = 2, class SYNC = BlockSync>
 __device__ __forceinline__ void grid_unit_xchg(float2* smem, int q, int V, int N, const float4* __restrict__ Z2,
                                                const int* __restrict__ gJ, const float2* __restrict__ gF,
@@ -787,20 +825,28 @@ __device__ __forceinline__ void grid_unit_xchg(float2* smem, int q, int V, int N
         x[2 * i + 1] = xo[i];
     }
     // the origin (row 0 of column q = 0, input 0 of thread 0, the gather gave 0
-    // there) is single-valued: mean over angles of the DC bin, by warp 0
-    if (live && q == 0 && tid < 32) {
-        float sx = 0.f, sy = 0.f;
-        for (int j = lane; j < V; j += 32) {
+    // there) is single-valued: mean over angles of the DC bin, by the block's threads
+    // through its lines, or, where the barrier covers other column pairs too, by warp 0
+    if (live && q == 0) {
+        using O = OriginSum<M, TPL>;
+        const auto dc = [&](int j) {
             const float4 zz = __ldg(Z2 + paired_slot(j, 0, H, V));
-            sx += zz.x;
-            sy += zz.y;
+            return make_float2(zz.x, zz.y);
+        };
+        if constexpr (std::is_same<SYNC, BlockSync>::value) {
+            const float2 part = O::warp(O::strided(dc, tid, V));
+            if (lane % O::W == 0) smem[tid / O::W] = part;
+            __syncthreads();
+            if (h == 0 && t == 0) {
+                float2 s = make_float2(0.f, 0.f);
+                for (int i = 0; i < 2 * TPL / O::W; ++i) s = cadd(s, smem[i]);
+                x[0] = make_float2(s.x / (float)V, s.y / (float)V);
+            }
+            __syncthreads();
+        } else if (tid < 32) {
+            const float2 s = O::by_warp(dc, lane, V);
+            if (lane == 0) x[0] = make_float2(s.x / (float)V, s.y / (float)V);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sx += __shfl_xor_sync(0xffffffffu, sx, o);
-            sy += __shfl_xor_sync(0xffffffffu, sy, o);
-        }
-        if (lane == 0) x[0] = make_float2(sx / (float)V, sy / (float)V);
     }
     const SmemLine sm{smem + h * smem_line_len(M)};
     const ColDst<NC> dst{Tp, N, M, h == 0 ? q : (q == 0 ? H : M - q), h == 1 && q != 0, live};

@@ -196,3 +196,25 @@ def test_captured_call(bst, N, V, S, chunk, warm, call):
         assert torch.equal(out, run(same, sino, torch.empty_like(out)))
     # the plan's streams serve calls outside the graph as before
     assert torch.equal(out, run(plan, sino, torch.empty_like(out)))
+
+
+# M = 32, 64, 128 (a column pair of less than a warp), 256 to 512 (groups of 8), 768, 1024 (of 4), 1536, 4096 (of 2)
+@pytest.mark.parametrize("N,V", [(16, 13), (32, 70), (64, 45), (48, 100), (128, 333), (192, 64), (256, 300), (384, 90),
+                                 (512, 100), (768, 75), (2048, 40)])
+def test_a_slice_does_not_depend_on_the_slices_beside_it(bst, N, V):
+    """Pairs of slices alone (paired kernels) and in whole groups (interleaved): the same volumes, bit for bit."""
+    gen = torch.Generator(device="cuda").manual_seed(N + V)
+    theta = synth.uniform_angles(V)
+    S = 4 * _group(2 * N)   # two groups
+    assert _grouped(2 * N, N, V, S) and not _grouped(2 * N, N, V, 2)
+    sino = torch.rand((S, V, N), device="cuda", generator=gen) + 0.5
+    flat = torch.full((S, N), 2.0, device="cuda")
+    plan = bst.Plan(N, theta, 2)
+    calls = (lambda s: plan.fbp(sino[s:s + 2]) if s is not None else plan.fbp(sino),
+             lambda s: plan.backproject(sino[s:s + 2]) if s is not None else plan.backproject(sino),
+             lambda s: plan.fbp_prep(sino[s:s + 2], flat=flat[s:s + 2], shift=1.5) if s is not None
+             else plan.fbp_prep(sino, flat=flat, shift=1.5))
+    for call in calls:
+        whole = call(None)
+        for s in range(0, S, 2):
+            assert torch.equal(call(s), whole[s:s + 2]), f"slices {s}, {s + 1}"
