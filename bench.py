@@ -118,11 +118,11 @@ KERNEL_SOURCES = ["paper_1704_08364_gb300/csrc/bst_forward.cuh", "paper_1704_083
                   "paper_1704_08364_gb300/csrc/bst_fft.cuh", "paper_1704_08364_gb300/csrc/bst_geo.cuh",
                   "paper_1704_08364_gb300/csrc/bst_inter.cuh"]
 CAPTURED_TRAFFIC = [
-    {"sha": "f2abd53a79b84892321685df4270eae8a0fdb8f438dc3e6e7abd891519d5e3dd",
+    {"sha": "3589eb27f673fec8429c26bb17d05e577f33495c9c18f71c3a869009b89fb8a7",
      "rays": 2048, "pad": 2,
      "shape": {"layout": "interleaved", "chunk_pairs": 16, "pair_fast": 1, "max_radix": 16, "grid_xchg": 1},
-     "bytes": {"k_ray_fft": 536984000 + 1018879000, "k_grid_col": 1147884000 + 1020602000,
-               "k_row_ifft": 1074021000 + 508716000}},
+     "bytes": {"k_ray_fft": 536986000 + 1018575000, "k_grid_col": 1148205000 + 1020441000,
+               "k_row_ifft": 1073890000 + 508508000}},
 ]
 
 

@@ -79,7 +79,8 @@ typedef enum {
 
 /* Launch shape of the forward path (extension; no passage: the paper fixes
  * the stages, not how they are tiled).  Results are identical up to
- * rounding whatever the shape. */
+ * rounding whatever the shape, and with one shape a slice's volume is the same
+ * bit for bit however many slices the call has (bilinear gridding). */
 typedef struct {
     int max_radix;    /* largest Stockham radix: 16 or 8 */
     int layout;       /* bst_layout_t */
@@ -219,7 +220,8 @@ size_t brute_workspace_bytes(bst_plan_t plan, int slices, int filtered);
  * d_g == NULL: plain B.  Otherwise each angle is first filtered along t with
  * h_k = |sigma_k| g[k] (h_0 = dsigma/4 g[0], h_{M/2} = 0) on the plan's padded
  * grid (SS filtered backprojection, x = B[F y]); the filtered sinogram goes
- * to d_ws (brute_workspace_bytes(plan, slices, 1) bytes).
+ * to d_ws (brute_workspace_bytes(plan, slices, 1) bytes).  The number of slices
+ * decides how many pixels a thread holds, which may change a slice's last bits.
  * Errors: INVALID_ARGUMENT, WORKSPACE_TOO_SMALL, CUDA. */
 bst_status_t brute_backproject(bst_plan_t plan, const float* d_sino, int slices,
                                const float* d_g, float* d_volume,
